@@ -78,11 +78,11 @@ typedef enum {
 #define MFBD_FLAG_SIMT_PROJECTION 0x2u /* FP32 phase projection and modal adjoint on the
                                         * SIMT kernels instead of the tensor cores
                                         * (comparison runs; not with MFBD_PREC_BF16_PHASE) */
-#define MFBD_FLAG_RECOMPUTE_BACKWARD 0x4u /* the adjoint recomputes the field F P and the
-                                           * pupil phasors instead of keeping them from
-                                           * the forward pass: 8 N^2 + 8 W^2 fewer bytes of
-                                           * device memory per (patch, object, frame), about
-                                           * 40 % more adjoint work */
+#define MFBD_FLAG_RECOMPUTE_BACKWARD 0x4u /* the adjoint recomputes the field F P instead of
+                                           * keeping it from the forward pass: 8 N^2 fewer
+                                           * bytes of device memory per (patch, object, frame)
+                                           * (at N = 64 also the 8 W^2 of the pupil phasors),
+                                           * about a quarter more adjoint work */
 #define MFBD_FLAG_GENERIC_KERNELS 0x8u /* run N = 64 on the kernels of the other patch
                                         * sizes (one CTA per unit) instead of the 64-pixel
                                         * pass machine (comparison runs) */

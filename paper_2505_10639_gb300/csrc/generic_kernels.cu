@@ -62,18 +62,17 @@ __global__ void loss_combine_kernel(const double* __restrict__ lpart, int S, dou
 
 }  // namespace
 
-size_t generic_smem(int N, int es, int es2, bool recompute) {
-    (void)es2;
-    (void)recompute;  // the recompute buffer is in global memory (e2scr)
-    return (size_t)N * es * sizeof(float2);
+size_t generic_smem(int N, bool half_box) {
+    const int stride = half_box ? N / 2 + 4 : N + 4;  // Geo<N>::S_HALF, S_FULL
+    return ((size_t)2 * N + (size_t)N * stride) * sizeof(float2);
 }
 
-int generic_adjoint_ctas(int N, int es, int sms) {
+int generic_adjoint_ctas(int N, bool half_box, int sms) {
     switch (N) {
-        case 48: return generic_adjoint_ctas_n<48>(es, sms);
-        case 64: return generic_adjoint_ctas_n<64>(es, sms);
-        case 96: return generic_adjoint_ctas_n<96>(es, sms);
-        case 128: return generic_adjoint_ctas_n<128>(es, sms);
+        case 48: return generic_adjoint_ctas_n<48>(half_box, sms);
+        case 64: return generic_adjoint_ctas_n<64>(half_box, sms);
+        case 96: return generic_adjoint_ctas_n<96>(half_box, sms);
+        case 128: return generic_adjoint_ctas_n<128>(half_box, sms);
         default: return 0;
     }
 }

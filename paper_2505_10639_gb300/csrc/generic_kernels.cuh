@@ -1,14 +1,14 @@
 // Pass kernels of one problem for patch sizes other than 64 (48, 96, 128),
 // and for 64 on request: one CTA per unit (patch, object, frame),
-// persistent over the units; for N <= 64 the CTA is one warp. The passes
-// themselves (Sec. 3.1, Eqs. 20-22 and their adjoint) are in unit_passes.cuh.
-// Each patch size is instantiated in a translation unit of its own
-// (generic_n48.cu ... generic_n128.cu) so that they compile in parallel.
+// persistent over the units. The passes themselves (Sec. 3.1, Eqs. 20-22 and
+// their adjoint) are in lane_passes.cuh. Each patch size is instantiated in a
+// translation unit of its own (generic_n48.cu ... generic_n128.cu) so that
+// they compile in parallel.
 #pragma once
 
 #include <algorithm>
 #include "mfbd_internal.h"
-#include "unit_passes.cuh"
+#include "lane_passes.cuh"
 
 namespace mfbd_dev {
 
@@ -16,7 +16,16 @@ namespace generic_detail {
 
 namespace {
 
-using namespace unitpass;
+using namespace lanepass;
+
+// CTAs per SM that the register budget is set for: two to three times 8 warps
+// at 80-128 registers a thread. Timed with one more and one less at each size
+// (forward / adjoint / recomputing adjoint, ms): 12,800 units of 128 px 0.735 /
+// 0.842 / 1.06 with 2 (0.787 / 1.018 / 1.23 with 3); 2,904 units of 96 px 0.111
+// / 0.131 / 0.165 with 3, 4, 3 (0.117 / 0.147 / 0.170 with 4, 3, 4); 48 px 0.193
+// / 0.215 with 12 (0.196 / 0.228 with 9).
+template <int N, bool ADJ, bool RECOMPUTE>
+constexpr int kMinCtas = N == 128 ? 2 : N == 96 ? (ADJ && !RECOMPUTE ? 4 : 3) : N == 64 ? 6 : 12;
 
 template <int N>
 __device__ __forceinline__ UnitPtr unit_ptr(const GenericParams& prm, long long u) {
@@ -32,56 +41,45 @@ __device__ __forceinline__ UnitPtr unit_ptr(const GenericParams& prm, long long 
     q.gphi = prm.gphi + ob.phi_off + img;
     q.h = prm.gscr + (size_t)u * N * Geo<N>::NH;
     q.pf = prm.pscr ? prm.pscr + (size_t)u * N * N : nullptr;
-    q.pp = prm.uscr ? prm.uscr + (size_t)u * prm.ustride : nullptr;
-    q.mask = ob.mask;
-    q.mw = ob.mw;
     q.W = ob.W;
     q.inv_z = ob.inv_z;
-    q.supp = ob.supp;
-    q.sw = prm.sw;
     q.cmask = ob.cmask;
     q.csupp = ob.csupp;
     return q;
 }
 
-// Threads of a CTA: N <= 64, one warp working on one unit at a time (32
-// lines per round, no CTA barrier); N = 96, 128, 128 threads on one unit (64
-// lines of two lanes per round).
+// Warps of a CTA: half of a pass's N / 8 groups of four lines, so that every
+// warp runs two of them.
 template <int N>
-struct Cta {
-    static constexpr bool WARP = N <= 64;
-    static constexpr int THREADS = WARP ? 32 : Geo<N>::THREADS;
-    static constexpr int LINES = WARP ? 32 : Geo<N>::LINES;
-    static constexpr int MIN_CTAS = WARP ? 12 : 1;  // 12 warps per SM: at most 170 registers a thread
-};
+constexpr int kWarps = N / 16;
 
-template <int N>
-__global__ void __launch_bounds__(Cta<N>::THREADS, Cta<N>::MIN_CTAS) generic_forward_kernel(const GenericParams prm) {
+template <int N, int S>
+__global__ void __launch_bounds__(32 * kWarps<N>, kMinCtas<N, false, false>) generic_forward_kernel(const GenericParams prm) {
     extern __shared__ __align__(16) unsigned char gsm[];
-    float2* E = reinterpret_cast<float2*>(gsm);
+    float2* tw = reinterpret_cast<float2*>(gsm);
+    float2* E = tw + 2 * N;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    load_twiddles<N>(tw, threadIdx.x, 32 * kWarps<N>);
+    __syncthreads();
     const long long units = (long long)prm.P * prm.K * prm.J;
-    for (long long u = blockIdx.x; u < units; u += gridDim.x) {
-        constexpr int L = Cta<N>::LINES;
-        if constexpr (Cta<N>::WARP) unit_forward_rounds<N, L>(unit_ptr<N>(prm, u), E, prm.es, threadIdx.x, WarpBar{});
-        else unit_forward<N, L>(unit_ptr<N>(prm, u), E, prm.es, threadIdx.x, CtaBar{});
-    }
+    for (long long u = blockIdx.x; u < units; u += gridDim.x)
+        unit_forward<N, S, kWarps<N>>(unit_ptr<N>(prm, u), E, tw, w, lane, CtaBar{});
 }
 
-template <int N, bool RECOMPUTE>
-__global__ void __launch_bounds__(Cta<N>::THREADS, Cta<N>::MIN_CTAS) generic_adjoint_kernel(const GenericParams prm) {
+template <int N, int S, bool RECOMPUTE>
+__global__ void __launch_bounds__(32 * kWarps<N>, kMinCtas<N, true, RECOMPUTE>) generic_adjoint_kernel(const GenericParams prm) {
     extern __shared__ __align__(16) unsigned char gsm[];
-    float2* E = reinterpret_cast<float2*>(gsm);
+    float2* tw = reinterpret_cast<float2*>(gsm);
+    float2* E = tw + 2 * N;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // RECOMPUTE: the column transforms of P, in this CTA's global buffer (kept
     // in L2) so that shared memory holds one exchange buffer
     float2* E2 = RECOMPUTE ? prm.e2scr + (size_t)blockIdx.x * N * prm.es2 : nullptr;
+    load_twiddles<N>(tw, threadIdx.x, 32 * kWarps<N>);
+    __syncthreads();
     const long long units = (long long)prm.P * prm.K * prm.J;
-    for (long long u = blockIdx.x; u < units; u += gridDim.x) {
-        constexpr int L = Cta<N>::LINES;
-        if constexpr (Cta<N>::WARP)
-            unit_adjoint<N, L, RECOMPUTE>(unit_ptr<N>(prm, u), E, prm.es, E2, prm.es2, threadIdx.x, WarpBar{});
-        else
-            unit_adjoint<N, L, RECOMPUTE>(unit_ptr<N>(prm, u), E, prm.es, E2, prm.es2, threadIdx.x, CtaBar{});
-    }
+    for (long long u = blockIdx.x; u < units; u += gridDim.x)
+        unit_adjoint<N, S, kWarps<N>, RECOMPUTE>(unit_ptr<N>(prm, u), E, E2, prm.es2, tw, w, lane, CtaBar{});
 }
 
 template <class Kern>
@@ -112,32 +110,48 @@ cudaError_t launch_persistent(Kern kern, int threads, size_t smem, long long uni
 
 }  // namespace generic_detail
 
+// f(integral constant of the buffer's row stride)
+template <int N, class F>
+auto with_stride(bool half_box, F&& f) {
+    using lanepass::Geo;
+    return half_box ? f(fftreg::IC<Geo<N>::S_HALF>{}) : f(fftreg::IC<Geo<N>::S_FULL>{});
+}
+
 template <int N>
-int generic_adjoint_ctas_n(int es, int sms) {
+int generic_adjoint_ctas_n(bool half_box, int sms) {
     using namespace generic_detail;
-    const size_t smem = generic_smem(N, es, 0, true);
-    long long c = 0;
-    const cudaError_t e = persistent_ctas(generic_adjoint_kernel<N, true>, Cta<N>::THREADS, smem, sms, &c);
-    return e == cudaSuccess ? (int)c : 0;
+    return with_stride<N>(half_box, [&](auto s) {
+        constexpr int S = decltype(s)::value;
+        long long c = 0;
+        const cudaError_t e = persistent_ctas(generic_adjoint_kernel<N, S, true>, 32 * kWarps<N>,
+                                              generic_smem(N, half_box), sms, &c);
+        return e == cudaSuccess ? (int)c : 0;
+    });
 }
 
 template <int N>
 cudaError_t launch_generic_forward_n(const GenericParams& prm, int sms, cudaStream_t s) {
     using namespace generic_detail;
     const long long units = (long long)prm.P * prm.K * prm.J;
-    const size_t smem = generic_smem(prm.N, prm.es, prm.es2, false);
-    return launch_persistent(generic_forward_kernel<N>, Cta<N>::THREADS, smem, units, sms, prm, s);
+    const size_t smem = generic_smem(N, prm.half_box);
+    return with_stride<N>(prm.half_box, [&](auto st) {
+        return launch_persistent(generic_forward_kernel<N, decltype(st)::value>, 32 * kWarps<N>, smem, units, sms, prm,
+                                 s);
+    });
 }
 
 template <int N>
 cudaError_t launch_generic_adjoint_n(const GenericParams& prm, int sms, cudaStream_t s) {
     using namespace generic_detail;
     const long long units = (long long)prm.P * prm.K * prm.J;
-    const bool rec = prm.pscr == nullptr;
-    const size_t smem = generic_smem(prm.N, prm.es, prm.es2, rec);
-    return rec ? launch_persistent(generic_adjoint_kernel<N, true>, Cta<N>::THREADS, smem, units, sms, prm, s,
-                                   prm.e2_ctas)
-               : launch_persistent(generic_adjoint_kernel<N, false>, Cta<N>::THREADS, smem, units, sms, prm, s);
+    const size_t smem = generic_smem(N, prm.half_box);
+    return with_stride<N>(prm.half_box, [&](auto st) {
+        constexpr int S = decltype(st)::value;
+        return prm.pscr == nullptr ? launch_persistent(generic_adjoint_kernel<N, S, true>, 32 * kWarps<N>, smem, units,
+                                                       sms, prm, s, prm.e2_ctas)
+                                   : launch_persistent(generic_adjoint_kernel<N, S, false>, 32 * kWarps<N>, smem,
+                                                       units, sms, prm, s);
+    });
 }
 
 }  // namespace mfbd_dev

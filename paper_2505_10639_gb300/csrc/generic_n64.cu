@@ -3,7 +3,7 @@
 
 namespace mfbd_dev {
 
-template int generic_adjoint_ctas_n<64>(int es, int sms);
+template int generic_adjoint_ctas_n<64>(bool half_box, int sms);
 template cudaError_t launch_generic_forward_n<64>(const GenericParams& prm, int sms, cudaStream_t s);
 template cudaError_t launch_generic_adjoint_n<64>(const GenericParams& prm, int sms, cudaStream_t s);
 

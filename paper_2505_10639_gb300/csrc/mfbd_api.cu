@@ -44,10 +44,8 @@ struct ObjectData {
     int g_chunk = 0, g_splits = 0;  // modal-adjoint pixel chunks for all P*J units (sizes part buffer)
     float* d_basis = nullptr;   // [M][W*W]
     uint64_t* d_mask = nullptr; // [W] box rows, then [N] box columns
-    uint32_t* d_gmask = nullptr;  // general sizes: [W][mw] box mask rows
     uint32_t* d_gsupp = nullptr;  // general sizes: [N][sw] OTF-support rows
     uint64_t* d_gcol = nullptr;   // general sizes: [W][2] box-column mask words, then [N/2+1][2] support columns
-    int mw = 0;
     uint64_t* d_supp = nullptr; // [N] rows, then [N] columns of the OTF support
     // tensor-core phase projection: the box basis as BF16 planes in the MMA
     // tile layout, [n_tiles][planes][Nt * Mp]; planes == 0: SIMT kernel
@@ -74,7 +72,8 @@ struct mfbd_plan {
     double* d_lpair = nullptr;  // its per-(patch, object) losses [P][K]
     int* d_lcnt = nullptr;      // its per-patch counts of finished objects [P], 0 between calls
     int* d_fticket = nullptr;   // its pair ticket and count of finished CTAs, 0 between calls
-    int es = 0, es2 = 0, sw = 0;  // their exchange-buffer strides and support-row words
+    bool half_box = false;      // every pupil box at most N/2 px: their smaller exchange buffer
+    int es2 = 0, sw = 0;        // row stride of e2scr's buffers, support-row words
     double gamma = 0;
     int* d_err = nullptr;       // set by a tensor-core kernel whose MMA wait gave up
     uint16_t* d_acoef = nullptr;  // coefficients as BF16 planes in the MMA tile layout
@@ -455,13 +454,11 @@ int run_generic(mfbd_plan_t p, int stages, const void* spectra, double* loss, vo
     const bool otf_only = (stages & ST_OTF_ONLY) != 0;
     g.gscr = otf_only ? gscr : p->d_gscr;
     g.pscr = otf_only ? nullptr : p->d_pscr;
-    g.uscr = otf_only ? nullptr : p->d_uscr;
-    g.ustride = p->ustride;
     g.spectra = static_cast<const float2*>(spectra);
     g.spec_ld = (p->flags & MFBD_FLAG_FULL_SPECTRUM) ? p->N : p->N / 2 + 1;
     g.loss = loss;
     g.object = static_cast<float2*>(object);
-    g.es = p->es;
+    g.half_box = p->half_box;
     g.es2 = p->es2;
     g.e2scr = p->d_e2scr;
     g.e2_ctas = p->e2_ctas;
@@ -474,8 +471,6 @@ int run_generic(mfbd_plan_t p, int stages, const void* spectra, double* loss, vo
         g.obj[k].W = o.W;
         g.obj[k].phi_off = o.phi_off + (long long)p0 * p->J * o.W * o.W;
         g.obj[k].inv_z = o.inv_z;
-        g.obj[k].mask = o.d_gmask;
-        g.obj[k].mw = o.mw;
         g.obj[k].supp = o.d_gsupp;
         g.obj[k].cmask = o.d_gcol;
         g.obj[k].csupp = o.d_gcol ? o.d_gcol + 2 * o.W : nullptr;
@@ -714,7 +709,7 @@ int mfbd_plan_create(mfbd_plan_t* out, const mfbd_plan_desc* d, void* stream) {
         if ((st = dev_alloc(p, &p->d_err, 1))) throw st;
         if ((e = cudaMemsetAsync(p->d_err, 0, sizeof(int), s))) throw cuda_fail(e, "clear error flag");
         std::vector<std::vector<uint64_t>> hm(p->K), hs(p->K);
-        std::vector<std::vector<uint32_t>> gm(p->K), gs(p->K);
+        std::vector<std::vector<uint32_t>> gs(p->K);
         std::vector<std::vector<uint64_t>> gc(p->K);
         long long phi_floats = 0;
         int max_box = 1;
@@ -766,13 +761,8 @@ int mfbd_plan_create(mfbd_plan_t* out, const mfbd_plan_desc* d, void* stream) {
                             hs[k][n + kx] |= 1ull << ky;
                         }
             } else {
-                // 32-bit words: box rows [W][mw], support rows [N][sw]
-                o.mw = (o.W + 31) / 32;
+                // 32-bit words: support rows [N][sw]
                 p->sw = (n / 2 + 1 + 31) / 32;
-                gm[k].assign((size_t)o.W * o.mw, 0u);
-                for (int yy = 0; yy < o.W; ++yy)
-                    for (int xx = 0; xx < o.W; ++xx)
-                        if (mask[(size_t)(o.x0 + yy) * n + (o.x0 + xx)]) gm[k][yy * o.mw + xx / 32] |= 1u << (xx % 32);
                 gs[k].assign((size_t)n * p->sw, 0u);
                 for (int ky = 0; ky < n; ++ky)
                     for (int kx = 0; kx <= n / 2; ++kx)
@@ -787,10 +777,8 @@ int mfbd_plan_create(mfbd_plan_t* out, const mfbd_plan_desc* d, void* stream) {
                 if ((st = dev_alloc(p, &o.d_gcol, gc[k].size()))) throw st;
                 if ((e = cudaMemcpyAsync(o.d_gcol, gc[k].data(), gc[k].size() * 8, cudaMemcpyHostToDevice, s)))
                     throw cuda_fail(e, "upload column masks");
-                if ((st = dev_alloc(p, &o.d_gmask, gm[k].size()))) throw st;
                 if ((st = dev_alloc(p, &o.d_gsupp, gs[k].size()))) throw st;
-                if ((e = cudaMemcpyAsync(o.d_gmask, gm[k].data(), gm[k].size() * 4, cudaMemcpyHostToDevice, s)) ||
-                    (e = cudaMemcpyAsync(o.d_gsupp, gs[k].data(), gs[k].size() * 4, cudaMemcpyHostToDevice, s)))
+                if ((e = cudaMemcpyAsync(o.d_gsupp, gs[k].data(), gs[k].size() * 4, cudaMemcpyHostToDevice, s)))
                     throw cuda_fail(e, "upload masks");
             }
             if ((st = dev_alloc(p, &o.d_basis, hb[k].size()))) throw st;
@@ -855,7 +843,7 @@ int mfbd_plan_create(mfbd_plan_t* out, const mfbd_plan_desc* d, void* stream) {
         if ((st = dev_alloc(p, &p->d_gscr, (size_t)p->P * p->K * p->J * n * (n / 2 + 1)))) throw st;
         if (keep && (st = dev_alloc(p, &p->d_pscr, (size_t)p->P * p->K * p->J * n * n))) throw st;
         p->ustride = (max_box * max_box + 31) & ~31;  // 256-byte aligned units
-        if (keep && (st = dev_alloc(p, &p->d_uscr, (size_t)p->P * p->K * p->J * p->ustride))) throw st;
+        if (keep && !p->generic && (st = dev_alloc(p, &p->d_uscr, (size_t)p->P * p->K * p->J * p->ustride))) throw st;
 
         p->sms = prop.multiProcessorCount;
         p->rsplit = reduction_split(p->P, p->K, n, p->sms);
@@ -882,13 +870,10 @@ int mfbd_plan_create(mfbd_plan_t* out, const mfbd_plan_desc* d, void* stream) {
                 }
             }
         } else {
-            // odd row strides: column accesses do not conflict in shared memory
-            p->es = std::max(n / 2 + 1, max_box) | 1;
-            p->es2 = max_box | 1;
-            if (generic_smem(n, p->es, p->es2, !keep) > (size_t)227 * 1024)
-                throw fail(MFBD_ERR_UNSUPPORTED, "the pupil box is too large for the shared-memory buffers");
+            p->half_box = max_box <= n / 2;
+            p->es2 = (max_box + 3) & ~3;  // rows start on 32-byte sectors
             if (!keep) {
-                p->e2_ctas = generic_adjoint_ctas(n, p->es, prop.multiProcessorCount);
+                p->e2_ctas = generic_adjoint_ctas(n, p->half_box, prop.multiProcessorCount);
                 if (p->e2_ctas < 1) throw fail(MFBD_ERR_UNSUPPORTED, "the adjoint kernel does not fit on this device");
                 if ((st = dev_alloc(p, &p->d_e2scr, (size_t)p->e2_ctas * n * p->es2))) throw st;
             }

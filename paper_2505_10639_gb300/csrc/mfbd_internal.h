@@ -168,8 +168,6 @@ struct GenericObj {
     int W;                  // side of the pupil's bounding box
     long long phi_off;      // float offset of this object's [P*J][W*W] phase block
     float inv_z;            // 1 / (N^2 n_pup)
-    const uint32_t* mask;   // [W][mw] box rows, bit c = pupil pixel at box column c
-    int mw;                 // words per mask row
     const uint32_t* supp;   // [N][sw] OTF support rows over kx <= N/2
     const uint64_t* cmask;  // [W][2] box columns: bit y = pupil pixel
     const uint64_t* csupp;  // [N/2+1][2] half-spectrum columns: bit ky = OTF support
@@ -183,14 +181,13 @@ struct GenericParams {
     const float* phi;       // box phases, per object at phi_off
     float* gphi;            // dL/dphi, same layout
     float2* gscr;           // [P][K][J][N][N/2+1]: OTF, then dL/dconj(H)
-    float2* pscr;           // [P][K][J][N x N] field p [x][y]; null: recomputed by the adjoint
-    float2* uscr;           // [P][K][J][ustride] pupil phasors; null: recomputed
-    int ustride;
+    float2* pscr;           // [P][K][J][N][N] field rows; null: recomputed by the adjoint
     const float2* spectra;  // D
     int spec_ld;            // N/2 + 1 or N
     double* loss;           // [P]
     float2* object;         // [P][K][N][spec_ld] or null
-    int es, es2;            // row strides (complex) of the exchange buffers
+    bool half_box;          // every pupil box at most N/2 px: the smaller exchange buffer
+    int es2;                // row stride (complex) of e2scr's buffers
     float2* e2scr;          // recompute: per-CTA second buffers [ctas][N * es2] in global memory (L2)
     int e2_ctas;            // CTAs e2scr has room for
     int rsplit;             // warps per (patch, object) of the frame reduction (<= 1: one)
@@ -200,15 +197,15 @@ struct GenericParams {
     GenericObj obj[kMaxObjects];
 };
 
-size_t generic_smem(int N, int es, int es2, bool recompute);
+size_t generic_smem(int N, bool half_box);
 // CTAs of the recompute adjoint launch on `sms` SMs (the size of e2scr).
-int generic_adjoint_ctas(int N, int es, int sms);
+int generic_adjoint_ctas(int N, bool half_box, int sms);
 cudaError_t launch_generic_forward(const GenericParams& prm, int sms, cudaStream_t s);
 cudaError_t launch_generic_reduction(const GenericParams& prm, int sms, cudaStream_t s);
 cudaError_t launch_generic_adjoint(const GenericParams& prm, int sms, cudaStream_t s);
 // The same per patch size, defined in generic_kernels.cuh and instantiated
 // in generic_n<N>.cu (one translation unit per size).
-template <int N> int generic_adjoint_ctas_n(int es, int sms);
+template <int N> int generic_adjoint_ctas_n(bool half_box, int sms);
 template <int N> cudaError_t launch_generic_forward_n(const GenericParams& prm, int sms, cudaStream_t s);
 template <int N> cudaError_t launch_generic_adjoint_n(const GenericParams& prm, int sms, cudaStream_t s);
 
