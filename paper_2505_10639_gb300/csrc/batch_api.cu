@@ -27,10 +27,9 @@ long long phi_stride(int W) { return round_up((long long)W * W, 64); }
 
 // Plan-time data shared by every (problem, object) with the same sampling.
 struct SharedObj {
-    int W = 0, x0 = 0, npup = 0, mw = 0, M = 0;
+    int W = 0, x0 = 0, npup = 0, M = 0;
     float* bm = nullptr;       // [M][W*W]
     float* bt = nullptr;       // [W*W][M]
-    uint32_t* mask = nullptr;  // [W][mw]
     uint32_t* supp = nullptr;  // [N][sw]
     uint64_t* cmask = nullptr; // [W][2] box columns
     uint64_t* csupp = nullptr; // [N/2+1][2] support columns
@@ -45,7 +44,7 @@ struct mfbd_batch {
     std::vector<long long> coeff_off, spec_off, loss_off, obj_off;
     long long coeff_floats = 0, spec_complex = 0, loss_doubles = 0, obj_complex = 0;
     long long patches = 0, units = 0;
-    int es_small = 33, es_large = 65;
+    bool half_box = true;               // every pupil box at most half its patch
     size_t smem = 0;
     int max_per_sm_v[2] = {0, 0};       // CTAs per SM of each kernel variant
     // schedule
@@ -92,7 +91,7 @@ void batch_release(mfbd_batch* b) {
 int unit_cost(int N) { return N * N; }
 
 // The item list of a schedule. Per patch: P, the F items (units k J + j in
-// fours when N <= 64), R, the A items, G. Staged: all P, all F, all R, all A, all
+// groups of kSmallUnits when N <= 64), R, the A items, G. Staged: all P, all F, all R, all A, all
 // G (each a launch). One launch: the patches are cut into windows of about
 // `window` 64 px units (0: one window) and window w's kind s goes into block
 // w + s, each block listing its older windows first, so an item's
@@ -112,10 +111,10 @@ std::vector<BatchItem> build_items(const mfbd_batch* b, int mode, int window, st
         it.prob = r.prob;
         it.patch = r.patch;
         if (kind == BK_FWD || kind == BK_ADJ) {
-            const int units = pr.K * pr.J;  // (k, j) flattened: a group of four may span two objects
+            const int units = pr.K * pr.J;  // (k, j) flattened: a group may span two objects
             for (int u = 0; u < units;) {
                 it.kj = u;
-                it.extra = pr.N <= 64 ? std::min(3, units - 1 - u) : 0;
+                it.extra = pr.N <= 64 ? std::min(kSmallUnits - 1, units - 1 - u) : 0;
                 out.push_back(it);
                 u += 1 + it.extra;
             }
@@ -209,8 +208,7 @@ int run_batch(mfbd_batch_t b, const float* coeffs, const void* spectra, double* 
     prm.probs = b->d_probs;
     prm.items = b->d_items;
     prm.kinds = kinds;
-    prm.es_small = b->es_small;
-    prm.es_large = b->es_large;
+    prm.half_box = b->half_box;
     prm.ctr = b->d_ctr;
     prm.err = b->d_ctr + ctr_ints;
     prm.coeffs = coeffs;
@@ -349,15 +347,10 @@ int mfbd_batch_create(mfbd_batch_t* out, const mfbd_plan_desc* problems, int n_p
                         hb[(size_t)m * npix + yy * W + xx] = v;
                         ht[(size_t)(yy * W + xx) * M + m] = v;
                     }
-            so.mw = (W + 31) / 32;
             const int sw = (n / 2 + 1 + 31) / 32;
-            const size_t mwords = (size_t)W * so.mw + (size_t)n * sw;
-            staging.emplace_back(mwords * sizeof(uint32_t), 0);
-            uint32_t* hm = reinterpret_cast<uint32_t*>(staging.back().data());
-            uint32_t* hs = hm + (size_t)W * so.mw;
-            for (int yy = 0; yy < W; ++yy)
-                for (int xx = 0; xx < W; ++xx)
-                    if (mask[(size_t)(lo + yy) * n + (lo + xx)]) hm[yy * so.mw + xx / 32] |= 1u << (xx % 32);
+            const size_t swords = (size_t)n * sw;
+            staging.emplace_back(swords * sizeof(uint32_t), 0);
+            uint32_t* hs = reinterpret_cast<uint32_t*>(staging.back().data());
             std::vector<uint8_t> sup = mfbd_host::otf_support_half(mask, n);
             for (int ky = 0; ky < n; ++ky)
                 for (int kx = 0; kx <= n / 2; ++kx)
@@ -365,9 +358,8 @@ int mfbd_batch_create(mfbd_batch_t* out, const mfbd_plan_desc* problems, int n_p
             if ((st = balloc(b, &so.bm, (size_t)2 * M * npix))) throw st;
             so.bt = so.bm + (size_t)M * npix;
             upload(hb, so.bm, (size_t)2 * M * npix * sizeof(float));
-            if ((st = balloc(b, &so.mask, mwords))) throw st;
-            so.supp = so.mask + (size_t)W * so.mw;
-            upload(hm, so.mask, mwords * sizeof(uint32_t));
+            if ((st = balloc(b, &so.supp, swords))) throw st;
+            upload(hs, so.supp, swords * sizeof(uint32_t));
             const size_t cwords = (size_t)2 * W + 2 * (n / 2 + 1);
             staging.emplace_back(cwords * sizeof(uint64_t), 0);
             uint64_t* hc = reinterpret_cast<uint64_t*>(staging.back().data());
@@ -389,7 +381,6 @@ int mfbd_batch_create(mfbd_batch_t* out, const mfbd_plan_desc* problems, int n_p
         b->loss_off.resize(n_problems);
         b->obj_off.resize(n_problems);
         long long gscr = 0, pscr = 0, phi = 0, ctr = 0;
-        int max_small = 0, max_large = 0;
         std::vector<std::vector<float>> weights(n_problems);
         std::vector<long long> w_off(n_problems);
         long long w_total = 0;
@@ -440,32 +431,27 @@ int mfbd_batch_create(mfbd_batch_t* out, const mfbd_plan_desc* problems, int n_p
                 }
                 BatchObj& ob = pr.obj[k];
                 ob.W = so.W;
-                ob.mw = so.mw;
                 ob.ldt = so.M;
                 ob.scale = (float)(d->wavelength[0] / d->wavelength[k]);
                 ob.inv_z = (float)(1.0 / ((double)n * n * so.npup));
                 ob.bm = so.bm;
                 ob.bt = so.bt;
-                ob.mask = so.mask;
                 ob.supp = so.supp;
                 ob.cmask = so.cmask;
                 ob.csupp = so.csupp;
                 ob.phi_koff = koff;
                 koff += (long long)pr.J * phi_stride(so.W);
-                if (n <= 64) max_small = std::max(max_small, so.W);
-                else max_large = std::max(max_large, so.W);
+                b->half_box = b->half_box && so.W <= n / 2;
             }
             pr.phi_patch = koff;
             pr.phi_off = phi;
             phi += (long long)pr.P * koff;
         }
-        b->es_small = std::max(33, max_small) | 1;
-        b->es_large = std::max(65, max_large) | 1;
-        b->smem = batch_smem(b->es_small, b->es_large);
-        if (b->smem > (size_t)227 * 1024)
-            throw set_error(MFBD_ERR_UNSUPPORTED, "a pupil box is too large for the batch kernel's shared memory");
-        b->max_per_sm_v[0] = batch_max_ctas_per_sm(b->smem, 0);
-        b->max_per_sm_v[1] = batch_max_ctas_per_sm(b->smem, 1);
+        bool sizes[4] = {};
+        for (const BatchProblem& pr : b->probs) sizes[pr.N == 48 ? 0 : pr.N / 32 - 1] = true;
+        b->smem = batch_smem(sizes, b->half_box);
+        b->max_per_sm_v[0] = batch_max_ctas_per_sm(b->smem, b->half_box, 0);
+        b->max_per_sm_v[1] = batch_max_ctas_per_sm(b->smem, b->half_box, 1);
         if (b->max_per_sm_v[0] < 1)
             throw set_error(MFBD_ERR_UNSUPPORTED, "the batch kernel does not fit on this device");
         // weights, problem table, scratch

@@ -17,13 +17,11 @@ int validate_desc(const mfbd_plan_desc* d);
 // One (problem, object): plan-time data on the device.
 struct BatchObj {
     int W;                  // side of the pupil's bounding box
-    int mw;                 // 32-bit words per box mask row
     int ldt;                // row stride of bt (>= M: bases are shared between problems)
     float scale;            // c_k = lambda_0 / lambda_k
     float inv_z;            // 1 / (N^2 n_pup)
     const float* bm;        // [M][W*W] basis on the box (0 outside the pupil)
     const float* bt;        // [W*W][ldt] the same, transposed
-    const uint32_t* mask;   // [W][mw] box rows
     const uint32_t* supp;   // [N][sw] OTF-support rows over kx <= N/2
     const uint64_t* cmask;  // [W][2] box columns: bit y = pupil pixel
     const uint64_t* csupp;  // [N/2+1][2] half-spectrum columns: bit ky = OTF support
@@ -48,8 +46,8 @@ struct BatchProblem {
     BatchObj obj[kMaxObjects];
 };
 
-// Work items. F and A cover one unit (patch, object, frame), or up to four
-// consecutive units k J + j of one patch when N <= 64 (one warp per unit);
+// Work items. F and A cover one unit (patch, object, frame), or several
+// consecutive units k J + j of one patch when N <= 64 (kSmallUnits);
 // P, R and G cover one patch.
 enum BatchKind : int {
     BK_PROJ = 0,   // phases of every object and frame of a patch (Eq. 22)
@@ -64,7 +62,7 @@ struct BatchItem {
     int prob;       // problem index
     int patch;      // patch within the problem
     int kj;         // F, A: k * J + j of the first unit; P, R, G: 0
-    int extra;      // F, A: further units kj + 1 .. kj + extra in the item (N <= 64: 0..3)
+    int extra;      // F, A: further units kj + 1 .. kj + extra in the item (N <= 64: 0 .. kSmallUnits - 1)
     int pad[3];
 };
 
@@ -78,7 +76,7 @@ struct BatchParams {
     int item0;              // first item of this launch (staged mode)
     int wait;               // 1: check dependencies (one launch over all kinds)
     int kinds;              // bit k set: items of kind k run (the others are skipped, and signalled)
-    int es_small, es_large; // exchange-buffer row strides (complex) for N <= 64 and N > 64
+    bool half_box;          // every pupil box at most N/2 px
     int* ctr;               // [patches][BC_COUNT] counters
     int* ticket;            // next item to take
     int* err;               // set when a dependency wait gives up
@@ -93,19 +91,23 @@ struct BatchParams {
     float* gphi;
 };
 
-constexpr int kBT = 128;  // threads per CTA of the batch kernel
-constexpr int kJC = 8;    // frames per register tile of its P and G items
+constexpr int kBT = 256;        // threads per CTA of the batch kernel
+constexpr int kJC = 8;          // frames per register tile of its P and G items
+constexpr int kSmallUnits = 2;  // units of an F or A item of N <= 64
+constexpr int kBatchTwiddles = 2 * (48 + 64 + 96 + 128);  // complex elements of the four tables
 
-size_t batch_smem(int es_small, int es_large);
-// Kernel variants: 0, a register budget of up to 255 a thread (2 CTAs per
-// SM); 1, up to 170 (3 CTAs per SM). Also sets the variant's dynamic
+// Dynamic shared memory for a batch holding the patch sizes (48, 64, 96, 128)
+// that are set in `sizes`.
+size_t batch_smem(const bool (&sizes)[4], bool half_box);
+// Kernel variants: 0, a register budget of up to 128 a thread (2 CTAs per
+// SM); 1, up to 80 (3 CTAs per SM). Also sets the variant's dynamic
 // shared-memory limit to `smem` (required before launch_batch).
-int batch_max_ctas_per_sm(size_t smem, int variant);
+int batch_max_ctas_per_sm(size_t smem, bool half_box, int variant);
 // One launch of `ctas` CTAs over items [item0, item0 + n_items).
 cudaError_t launch_batch(const BatchParams& prm, int ctas, size_t smem, int variant, cudaStream_t s);
 // The same per register budget (MINB CTAs per SM), defined in
 // batch_kernels.cuh and instantiated in batch_kernel_v2.cu / batch_kernel_v3.cu.
-template <int MINB> int batch_max_ctas_variant(size_t smem);
+template <int MINB> int batch_max_ctas_variant(size_t smem, bool half_box);
 template <int MINB> cudaError_t launch_batch_variant(const BatchParams& prm, int ctas, size_t smem, cudaStream_t s);
 
 }  // namespace mfbd_dev

@@ -6,16 +6,18 @@
 
 namespace mfbd_dev {
 
-size_t batch_smem(int es_small, int es_large) {
-    // four 64-pixel warps, one 128-pixel unit, or the P item's coefficient tile
-    const size_t small = (size_t)(kBT / 32) * 64 * es_small * sizeof(float2);
-    const size_t large = (size_t)128 * es_large * sizeof(float2);
-    const size_t proj = (size_t)kJC * 256 * sizeof(float);
-    return std::max(std::max(small, large), proj);
+size_t batch_smem(const bool (&sizes)[4], bool half_box) {
+    // the twiddles, then the exchange buffers of an item or the P item's coefficient tile
+    size_t unit = kJC * 256 * sizeof(float) / sizeof(float2);
+    const int n[4] = {48, 64, 96, 128};
+    for (int i = 0; i < 4; ++i)
+        if (sizes[i])
+            unit = std::max(unit, (size_t)(n[i] <= 64 ? kSmallUnits : 1) * n[i] * (half_box ? n[i] / 2 + 4 : n[i] + 4));
+    return (kBatchTwiddles + unit) * sizeof(float2);
 }
 
-int batch_max_ctas_per_sm(size_t smem, int variant) {
-    return variant == 1 ? batch_max_ctas_variant<3>(smem) : batch_max_ctas_variant<2>(smem);
+int batch_max_ctas_per_sm(size_t smem, bool half_box, int variant) {
+    return variant == 1 ? batch_max_ctas_variant<3>(smem, half_box) : batch_max_ctas_variant<2>(smem, half_box);
 }
 
 cudaError_t launch_batch(const BatchParams& prm, int ctas, size_t smem, int variant, cudaStream_t s) {

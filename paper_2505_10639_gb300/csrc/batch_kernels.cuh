@@ -7,7 +7,7 @@
 // F, the forward passes of a unit (Eqs. 20-21 and the OTF); R, the frame
 // reduction of a patch (Sec. 2.2.1, Eqs. 11-12, and the adjoint seeds); A,
 // the adjoint passes of a unit (-> dL/dphi); G, the modal adjoint of a patch
-// (dL/da = sum_k c_k B_k^T dL/dphi_k). CTAs (128 threads) take items in list
+// (dL/da = sum_k c_k B_k^T dL/dphi_k). CTAs (256 threads) take items in list
 // order from a ticket counter. In one-launch mode an item first waits for
 // the items it depends on (P -> F -> R -> A -> G of the same patch), which
 // all come earlier in the list: the holder of the smallest unfinished ticket
@@ -16,13 +16,13 @@
 // the host launches each kind's range of the list separately and nothing
 // waits.
 //
-// F and A items of patches of N <= 64 px cover up to four consecutive units
-// (k J + j) of one patch: each of the CTA's four warps runs one unit on its own
-// exchange buffer with warp synchronisation only. Larger patches use all 128
-// threads on one unit. Every pass runs as rounds with one register FFT per
-// (patch size, direction) (unit_forward_rounds, unit_adjoint_rounds): the
-// kernel holds all patch sizes and both directions, and the smaller code was
-// measured faster here (18.7 against 20.7 ms on the 2000-problem batch).
+// F and A items of patches of N <= 64 px cover up to two consecutive units
+// (k J + j) of one patch: four warps run one unit each on their own exchange
+// buffer and named barrier. Larger patches use all eight warps on one unit.
+// The passes are those of lane_passes.cuh. Measured on 500 drawn problems
+// (15,788 units): 6.76 ms with a unit per warp (N <= 64) or per 128 threads
+// and one or two lanes a line, 3.59 ms with these; F 1.17 -> 0.52, A 1.52 ->
+// 0.70 ms of the staged schedule.
 //
 // Data written by one CTA and read by another inside the launch (phases,
 // OTFs and seeds, fields, dL/dphi) is published by the writer's barrier,
@@ -37,7 +37,8 @@
 #pragma once
 
 #include "batch_internal.h"
-#include "unit_passes.cuh"
+#include "frame_reduction.cuh"
+#include "lane_passes.cuh"
 
 #include <algorithm>
 
@@ -46,7 +47,8 @@ namespace mfbd_dev {
 
 namespace {
 
-using namespace unitpass;
+using namespace lanepass;
+using namespace reduction;
 
 constexpr long long kSpinLimit = 1ll << 22; // polls of a dependency counter (~1 s)
 
@@ -84,38 +86,45 @@ __device__ __forceinline__ UnitPtr batch_unit(const BatchParams& prm, const Batc
     q.gphi = prm.gphi + phi;
     q.h = prm.gscr + pr.gscr_off + u * N * Geo<N>::NH;
     q.pf = prm.pscr + pr.pscr_off + u * N * N;
-    q.pp = nullptr;  // exp(i phi) is recomputed from the phase in the adjoint
-    q.mask = ob.mask;
-    q.mw = ob.mw;
     q.W = ob.W;
     q.inv_z = ob.inv_z;
-    q.supp = ob.supp;
-    q.sw = pr.sw;
     q.cmask = ob.cmask;
     q.csupp = ob.csupp;
     return q;
 }
 
-// F or A item: one unit per warp (N <= 64: up to four units of one patch,
-// 32 lines per round, warp synchronisation only) or one unit on the
-// whole CTA (N = 96, 128: 64 lines of two lanes per round, CTA barriers).
-template <int N, bool ADJ>
-__device__ void item_unit(const BatchParams& prm, const BatchProblem& pr, const BatchItem& it, float2* smem) {
-    const int t = threadIdx.x;
-    if constexpr (N <= 64) {
-        const int w = t >> 5, lane = t & 31;
-        if (w > it.extra) return;
-        const int kj = it.kj + w, k = kj / pr.J, j = kj - k * pr.J;
-        const UnitPtr q = batch_unit<N>(prm, pr, it.patch, k, j);
-        float2* E = smem + (size_t)w * N * prm.es_small;
-        if constexpr (ADJ) unit_adjoint_rounds<N, 32, false>(q, E, prm.es_small, nullptr, 0, lane, WarpBar{});
-        else unit_forward_rounds<N, 32>(q, E, prm.es_small, lane, WarpBar{});
-    } else {
-        const int k = it.kj / pr.J, j = it.kj - k * pr.J;
-        const UnitPtr q = batch_unit<N>(prm, pr, it.patch, k, j);
-        if constexpr (ADJ) unit_adjoint_rounds<N, 64, false>(q, smem, prm.es_large, nullptr, 0, t, CtaBar{});
-        else unit_forward_rounds<N, 64>(q, smem, prm.es_large, t, CtaBar{});
+// Barrier of a group of `n` threads (a multiple of 32) on named barrier `id`.
+struct GroupBar {
+    int id, n;
+    __device__ __forceinline__ void operator()() const {
+        asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
     }
+};
+
+// Twiddles of every patch size, one after the other at the start of the
+// CTA's shared memory (complex elements).
+template <int N>
+constexpr int kTwOff = N == 48 ? 0 : N == 64 ? 96 : N == 96 ? 224 : 416;
+static_assert(kTwOff<128> + 2 * 128 == kBatchTwiddles, "room for the four tables");
+
+// F or A item: two units of one patch, four warps each (N <= 64), or one unit
+// on the whole CTA (N = 96, 128).
+template <int N, bool HALF, bool ADJ>
+__device__ void item_unit(const BatchParams& prm, const BatchProblem& pr, const BatchItem& it, float2* smem) {
+    constexpr int S = HALF ? Geo<N>::S_HALF : Geo<N>::S_FULL;
+    constexpr int kUnits = N <= 64 ? kSmallUnits : 1, kW = kBT / 32 / kUnits;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, g = w / kW;
+    if (g > it.extra) return;
+    const int kj = it.kj + g, k = kj / pr.J, j = kj - k * pr.J;
+    const UnitPtr q = batch_unit<N>(prm, pr, it.patch, k, j);
+    const float2* tw = smem + kTwOff<N>;
+    float2* E = smem + kBatchTwiddles + (size_t)g * N * S;
+    auto run = [&](auto bar) {
+        if constexpr (ADJ) unit_adjoint<N, S, kW, false>(q, E, nullptr, 0, tw, w - g * kW, lane, bar);
+        else unit_forward<N, S, kW>(q, E, tw, w - g * kW, lane, bar);
+    };
+    if constexpr (kUnits > 1) run(GroupBar{1 + g, 32 * kW});
+    else run(CtaBar{});
 }
 
 // P item: phi_kj[i] = c_k sum_m a_j[m] B_k[m][i] on every box pixel i, for
@@ -216,8 +225,8 @@ __device__ void item_grad(const BatchParams& prm, const BatchProblem& pr, int p)
     }
 }
 
-// R item: the four warps share each object's frequencies (warp w takes
-// f = 32 w + lane + 128 i); the patch loss adds the warps' sums of an object
+// R item: the CTA's warps share each object's frequencies (warp w takes
+// f = 32 w + lane + kBT i); the patch loss adds the warps' sums of an object
 // in warp order, then the objects in order.
 __device__ void item_reduce(const BatchParams& prm, const BatchProblem& pr, int p, double* sobj) {
     constexpr int kW = kBT / 32;
@@ -252,23 +261,28 @@ __device__ void item_reduce(const BatchParams& prm, const BatchProblem& pr, int 
     }
 }
 
-template <bool ADJ>
+template <bool HALF, bool ADJ>
 __device__ void dispatch_unit(const BatchParams& prm, const BatchProblem& pr, const BatchItem& it, float2* smem) {
     switch (pr.N) {
-        case 48: item_unit<48, ADJ>(prm, pr, it, smem); break;
-        case 64: item_unit<64, ADJ>(prm, pr, it, smem); break;
-        case 96: item_unit<96, ADJ>(prm, pr, it, smem); break;
-        default: item_unit<128, ADJ>(prm, pr, it, smem); break;
+        case 48: item_unit<48, HALF, ADJ>(prm, pr, it, smem); break;
+        case 64: item_unit<64, HALF, ADJ>(prm, pr, it, smem); break;
+        case 96: item_unit<96, HALF, ADJ>(prm, pr, it, smem); break;
+        default: item_unit<128, HALF, ADJ>(prm, pr, it, smem); break;
     }
 }
 
-// MINB: CTAs per SM the register budget is set for (2: up to 255 registers a
-// thread; 3: up to 170, the 96 and 128 px passes then spill). The autotuner
-// picks one.
-template <int MINB>
+// MINB: CTAs per SM the register budget is set for (2: up to 128 registers a
+// thread; 3: up to 80). The autotuner picks one. HALF: every pupil box of the
+// batch is at most half its patch, and the exchange buffers are the half-box
+// ones.
+template <int MINB, bool HALF>
 __global__ void __launch_bounds__(kBT, MINB) batch_kernel(const BatchParams prm) {
     extern __shared__ __align__(16) unsigned char bsm[];
     float2* smem = reinterpret_cast<float2*>(bsm);
+    load_twiddles<48>(smem + kTwOff<48>, threadIdx.x, kBT);
+    load_twiddles<64>(smem + kTwOff<64>, threadIdx.x, kBT);
+    load_twiddles<96>(smem + kTwOff<96>, threadIdx.x, kBT);
+    load_twiddles<128>(smem + kTwOff<128>, threadIdx.x, kBT);
     __shared__ int s_item, s_ok;
     __shared__ double sobj[kMaxObjects * (kBT / 32)];
     for (;;) {
@@ -296,10 +310,10 @@ __global__ void __launch_bounds__(kBT, MINB) batch_kernel(const BatchParams prm)
         __syncthreads();
         if (s_ok && ((prm.kinds >> it.kind) & 1)) {
             switch (it.kind) {
-                case BK_PROJ: item_proj(prm, pr, it.patch, reinterpret_cast<float*>(bsm)); break;
-                case BK_FWD: dispatch_unit<false>(prm, pr, it, smem); break;
+                case BK_PROJ: item_proj(prm, pr, it.patch, reinterpret_cast<float*>(smem + kBatchTwiddles)); break;
+                case BK_FWD: dispatch_unit<HALF, false>(prm, pr, it, smem); break;
                 case BK_RED: item_reduce(prm, pr, it.patch, sobj); break;
-                case BK_ADJ: dispatch_unit<true>(prm, pr, it, smem); break;
+                case BK_ADJ: dispatch_unit<HALF, true>(prm, pr, it, smem); break;
                 default: item_grad(prm, pr, it.patch); break;
             }
         }
@@ -317,19 +331,18 @@ __global__ void __launch_bounds__(kBT, MINB) batch_kernel(const BatchParams prm)
 }  // namespace
 
 template <int MINB>
-int batch_max_ctas_variant(size_t smem) {
-    if (cudaFuncSetAttribute(batch_kernel<MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-        return 0;
+int batch_max_ctas_variant(size_t smem, bool half_box) {
+    auto kern = half_box ? batch_kernel<MINB, true> : batch_kernel<MINB, false>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<MINB>, kBT, smem) != cudaSuccess)
-        return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kBT, smem) != cudaSuccess) return 0;
     return per_sm;
 }
 
 template <int MINB>
 cudaError_t launch_batch_variant(const BatchParams& prm, int ctas, size_t smem, cudaStream_t s) {
-    batch_kernel<MINB><<<ctas, kBT, smem, s>>>(prm);
+    if (prm.half_box) batch_kernel<MINB, true><<<ctas, kBT, smem, s>>>(prm);
+    else batch_kernel<MINB, false><<<ctas, kBT, smem, s>>>(prm);
     return cudaGetLastError();
 }
 

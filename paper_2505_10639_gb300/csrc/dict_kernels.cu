@@ -26,7 +26,7 @@
 // frame order; the patch loss = the units' losses summed over (k, j) in order.
 #include "../../include/mfbd.h"
 #include "mfbd_internal.h"
-#include "unit_passes.cuh"
+#include "line_fft.cuh"
 
 #include <cuda_runtime.h>
 
@@ -36,7 +36,7 @@ using namespace mfbd_dev;
 
 namespace {
 
-using namespace mfbd_dev::unitpass;
+using namespace mfbd_dev::linefft;
 
 constexpr int kDN = 64, kDNH = kDN / 2 + 1, kDES = kDNH;  // exchange stride 33 (odd)
 constexpr int kDoLd = kDN + 1;                             // dL/do rows, padded

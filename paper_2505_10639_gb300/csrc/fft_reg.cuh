@@ -95,11 +95,9 @@ constexpr int bitrev(int i) {
 
 // Complex add and subtract. On sm_100 and later each is one paired FP32
 // instruction (FADD2: two round-to-nearest adds, the same results as two
-// scalar adds) instead of two: the butterflies issue fewer instructions. A
-// translation unit that defines MFBD_SCALAR_COMPLEX_ADD before including
-// this header keeps the scalar adds (the batch kernel, measured 3 % faster
-// with them; the 128 px field 3 % faster with the paired ones).
-#if defined(__CUDA_ARCH__) && (__CUDA_ARCH__ >= 1000) && !defined(MFBD_SCALAR_COMPLEX_ADD)
+// scalar adds) instead of two: the butterflies issue fewer instructions (the
+// 128 px field 3 % faster, the batch kernel 1.5 %).
+#if defined(__CUDA_ARCH__) && (__CUDA_ARCH__ >= 1000)
 #define MFBD_PAIRED_ADD 1
 #endif
 MFBD_HD float2 cadd(float2 a, float2 b) {

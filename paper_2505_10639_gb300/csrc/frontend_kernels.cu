@@ -34,7 +34,7 @@
 // cosf.
 #include "mfbd_internal.h"
 #include "tma.cuh"
-#include "unit_passes.cuh"
+#include "line_fft.cuh"
 
 #include <cmath>
 
@@ -42,7 +42,7 @@ namespace mfbd_dev {
 
 namespace {
 
-using namespace unitpass;
+using namespace linefft;
 
 // Threads per CTA: one warp for N <= 64 (32 lines per round, every lane
 // busy in the N/2-line passes), 128 for N = 96, 128 (64 lines of two lanes).

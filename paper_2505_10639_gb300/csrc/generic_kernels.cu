@@ -4,13 +4,13 @@
 #include <algorithm>
 
 #include "mfbd_internal.h"
-#include "unit_passes.cuh"
+#include "frame_reduction.cuh"
 
 namespace mfbd_dev {
 
 namespace {
 
-using namespace unitpass;
+using namespace reduction;
 
 // One CTA per patch (persistent over patches), one warp per object; the
 // patch loss sums the objects in order.

@@ -28,3 +28,32 @@ def test_pupil_box_edges(n_pix, diams, recompute):
     assert plan.info()["slots_per_cta"] == 0  # the general-size kernels
     loss, grad, obj = _run_fused(plan, a32, d32)
     _check(case, loss, grad, obj, _oracle(case, a32, d_or))
+
+
+@pytest.mark.parametrize("shapes", [
+    [(48, 24.0, 3)],                                                     # one small size: the smallest buffer
+    [(48, 26.0, 1), (64, 64.0, 2), (96, 50.0, 3), (128, 66.0, 2)],       # boxes wider than half: the full-box buffer
+    [(48, 20.0, 2), (64, 32.0, 5), (96, 48.0, 1), (128, 64.0, 3)],       # odd unit counts, boxes of exactly half
+])
+def test_batch_box_and_unit_edges(shapes):
+    """Uneven batches whose units do not fill their items, against plans of the single problems."""
+    import torch
+
+    from paper_2505_10639_gb300.mfbd import Batch, Problem
+    data = []
+    for i, (n, diam, frames) in enumerate(shapes):
+        case = cases.make_case(n_pix=n, diams=(diam,), wavelengths=(6563.0,), n_frames=frames, n_modes=6,
+                               basis="zernike", n_patches=1, seed=20250700 + i)
+        a32, d32, d_or = _inputs(case)
+        data.append((case, a32, d32, _oracle(case, a32, d_or)))
+    b = Batch([Problem(c["n_pix"], 1, c["diams"], c["wavelengths"], c["n_frames"], c["n_modes"],
+                       gamma=c["setup"].gamma) for c, _, _, _ in data])
+    coeffs = Batch.pack([torch.from_numpy(a).cuda() for _, a, _, _ in data])
+    spectra = Batch.pack([torch.from_numpy(d).cuda() for _, _, d, _ in data])
+    for variant in (0, 1):
+        b.set_schedule("one_launch", 0, 0, variant)
+        out = b.loss_grad(coeffs, spectra, want_object=True)
+        b.check()
+        loss, grad, obj = (b.unpack(t, k) for t, k in zip(out, ("loss", "grad", "object")))
+        for i, (case, _, _, ref) in enumerate(data):
+            _check(case, loss[i].cpu().numpy(), grad[i].cpu().numpy(), obj[i].cpu().numpy().astype("complex128"), ref)
