@@ -94,7 +94,7 @@ struct BatchParams {
 constexpr int kBT = 256;        // threads per CTA of the batch kernel
 constexpr int kJC = 8;          // frames per register tile of its P and G items
 constexpr int kSmallUnits = 2;  // units of an F or A item of N <= 64
-constexpr int kBatchTwiddles = 2 * (48 + 64 + 96 + 128);  // complex elements of the four tables
+constexpr int kBatchTwiddles = 96 + 64 + 192 + 128;  // complex elements of the four tables
 
 // Dynamic shared memory for a batch holding the patch sizes (48, 64, 96, 128)
 // that are set in `sizes`.

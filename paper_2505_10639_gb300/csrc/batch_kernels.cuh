@@ -104,8 +104,9 @@ struct GroupBar {
 // Twiddles of every patch size, one after the other at the start of the
 // CTA's shared memory (complex elements).
 template <int N>
-constexpr int kTwOff = N == 48 ? 0 : N == 64 ? 96 : N == 96 ? 224 : 416;
-static_assert(kTwOff<128> + 2 * 128 == kBatchTwiddles, "room for the four tables");
+constexpr int kTwOff = N == 48 ? 0 : N == 64 ? 96 : N == 96 ? 160 : 352;
+static_assert(kTwOff<64> == Twiddles<48>::kElems && kTwOff<96> == kTwOff<64> + Twiddles<64>::kElems &&
+                  kTwOff<128> == kTwOff<96> + Twiddles<96>::kElems && kTwOff<128> + Twiddles<128>::kElems == kBatchTwiddles, "room for the four tables");
 
 // F or A item: two units of one patch, four warps each (N <= 64), or one unit
 // on the whole CTA (N = 96, 128).
@@ -121,7 +122,8 @@ __device__ void item_unit(const BatchParams& prm, const BatchProblem& pr, const 
     float2* E = smem + kBatchTwiddles + (size_t)g * N * S;
     auto run = [&](auto bar) {
         if constexpr (ADJ) unit_adjoint<N, S, kW, false>(q, E, nullptr, 0, tw, w - g * kW, lane, bar);
-        else unit_forward<N, S, kW>(q, E, tw, w - g * kW, lane, bar);
+        else if ((prm.kinds >> BK_RED) & 1) unit_forward<N, S, kW, false>(q, E, tw, w - g * kW, lane, bar);
+        else unit_forward<N, S, kW, true>(q, E, tw, w - g * kW, lane, bar);  // the OTFs alone
     };
     if constexpr (kUnits > 1) run(GroupBar{1 + g, 32 * kW});
     else run(CtaBar{});
@@ -225,14 +227,13 @@ __device__ void item_grad(const BatchParams& prm, const BatchProblem& pr, int p)
     }
 }
 
-// R item: the CTA's warps share each object's frequencies (warp w takes
-// f = 32 w + lane + kBT i); the patch loss adds the warps' sums of an object
-// in warp order, then the objects in order.
-__device__ void item_reduce(const BatchParams& prm, const BatchProblem& pr, int p, double* sobj) {
-    constexpr int kW = kBT / 32;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// R item: the CTA's threads share each object's frequencies; the patch loss
+// adds an object's warps in order, then the objects in order.
+template <int HOLD>
+__device__ void item_reduce(const BatchParams& prm, const BatchProblem& pr, int p, double* part) {
     const int N = pr.N, NH = N / 2 + 1, J = pr.J;
     const size_t dstride = (size_t)N * NH;
+    double tot = 0.0;
     for (int k = 0; k < pr.K; ++k) {
         const size_t unit0 = ((size_t)p * pr.K + k) * J;
         RedPtr r;
@@ -246,19 +247,10 @@ __device__ void item_reduce(const BatchParams& prm, const BatchProblem& pr, int 
         r.supp = pr.obj[k].supp;
         r.sw = pr.sw;
         r.obj = prm.object ? prm.object + pr.obj_off + ((size_t)p * pr.K + k) * dstride : nullptr;
-        const double v = reduce_warp(r, lane, 32 * warp, 32 * kW);
-        if (lane == 0) sobj[k * kW + warp] = v;
+        tot += cta_sum<kBT / 32>(reduce_lane<HOLD>(r, threadIdx.x, kBT), part);
+        __syncthreads();
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int k = 0; k < pr.K; ++k) {
-            double tk = 0.0;
-            for (int w = 0; w < kW; ++w) tk += sobj[k * kW + w];
-            tot += tk;
-        }
-        prm.loss[pr.loss_off + p] = tot;
-    }
+    if (threadIdx.x == 0) prm.loss[pr.loss_off + p] = tot;
 }
 
 template <bool HALF, bool ADJ>
@@ -284,7 +276,7 @@ __global__ void __launch_bounds__(kBT, MINB) batch_kernel(const BatchParams prm)
     load_twiddles<96>(smem + kTwOff<96>, threadIdx.x, kBT);
     load_twiddles<128>(smem + kTwOff<128>, threadIdx.x, kBT);
     __shared__ int s_item, s_ok;
-    __shared__ double sobj[kMaxObjects * (kBT / 32)];
+    __shared__ double part[kBT / 32];
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(prm.ticket, 1);
         __syncthreads();
@@ -312,7 +304,7 @@ __global__ void __launch_bounds__(kBT, MINB) batch_kernel(const BatchParams prm)
             switch (it.kind) {
                 case BK_PROJ: item_proj(prm, pr, it.patch, reinterpret_cast<float*>(smem + kBatchTwiddles)); break;
                 case BK_FWD: dispatch_unit<HALF, false>(prm, pr, it, smem); break;
-                case BK_RED: item_reduce(prm, pr, it.patch, sobj); break;
+                case BK_RED: item_reduce<MINB == 2 ? 16 : 8>(prm, pr, it.patch, part); break;
                 case BK_ADJ: dispatch_unit<HALF, true>(prm, pr, it, smem); break;
                 default: item_grad(prm, pr, it.patch); break;
             }

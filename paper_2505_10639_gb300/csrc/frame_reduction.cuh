@@ -21,11 +21,10 @@ __device__ __forceinline__ bool wbit(const uint32_t* rows, int words, int r, int
     return (rows[r * words + (c >> 5)] >> (c & 31)) & 1u;
 }
 
-// Frame reduction of one (patch, object) by one warp, any patch size: the
-// residual form of Eq. 12 in FP32 with FP64 where it would cancel, Kahan sums
-// per lane and an FP64 warp combine; writes the object (Eq. 11) when `obj`
-// is not null and the adjoint seeds G_j = -w_j conj(O) (D_j - O H_j) over H_j.
-// Returns the (patch, object) loss on every lane.
+// Frame reduction of one (patch, object), any patch size: the residual form of
+// Eq. 12 in FP32 with FP64 where it would cancel, Kahan sums per lane; writes
+// the object (Eq. 11) when `obj` is not null and the adjoint seeds
+// G_j = -w_j conj(O) (D_j - O H_j) over H_j.
 struct RedPtr {
     int N, J, spec_ld;      // spectra / object row stride: N/2 + 1 or N
     double gamma;
@@ -39,71 +38,134 @@ struct RedPtr {
     float2* gobj = nullptr;          // with oin: dL/dconj(O) [N][spec_ld], or null
 };
 
-// Lanes take the frequencies f0 + lane, f0 + lane + fstep, ... (fstep a
-// multiple of 32: several warps can share one (patch, object)); the returned
-// sum covers this warp's frequencies.
-__device__ __forceinline__ double reduce_warp(const RedPtr& r, int lane, int f0 = 0, int fstep = 32) {
+// Lanes take the frequencies f0, f0 + fstep, ...; the returned sum covers
+// this lane's. Outside the OTF support H vanishes and G with it: neither is
+// read or written there (the passes of the larger sizes do not store or load
+// them either), which at pupils of 0.35 to 0.5 N px leaves 40 to 80 % of the
+// half spectrum.
+//
+// HBM is the floor (D once, H and G once on the support); what it needs is
+// loads in flight. For J <= HOLD a frequency's frames are loaded once, all at
+// once, into registers; otherwise in chunks of kChunk frames, twice (the second
+// time from L2). Lanes outside the support take the same way with their loads
+// of H predicated off: a path of their own, which most warps would run as well
+// as the other, was slower (96 px 0.081 -> 0.100 ms).
+template <int HOLD>
+__device__ __forceinline__ double reduce_lane(const RedPtr& r, int f0, int fstep) {
+    constexpr int kChunk = 8;
     const int N = r.N, NH = N / 2 + 1, half = N * NH, J = r.J;
-    const size_t dstride = (size_t)N * r.spec_ld;
+    const unsigned dstride = (unsigned)N * r.spec_ld;  // J * dstride < 2^32
     const float gam = (float)r.gamma;
     KahanSum acc;
-    for (int f = f0 + lane; f < half; f += fstep) {
+    for (int f = f0; f < half; f += fstep) {
         const int ky = f / NH, kx = f - ky * NH;
         const size_t doff = (size_t)ky * r.spec_ld + kx;
         const float2* dp = r.d + doff;
         float2* hp = r.h + f;
-        const bool seed = (f != 0) && wbit(r.supp, r.sw, ky, kx);
-        if (r.oin) {  // object-inferring loss: the object is given
-            float2 g;
-            const float t = explicit_frequency(J, dp, dstride, hp, half, r.w, r.gamma, seed, r.oin[doff], g);
-            acc.add((kx == 0 || kx == N / 2) ? t : 2.0f * t);
-            if (r.gobj) {
-                r.gobj[doff] = g;
-                if (r.spec_ld == N && kx > 0 && kx < N / 2) r.gobj[(size_t)((N - ky) % N) * N + (N - kx)] = cconj(g);
-            }
-            continue;
-        }
-        float2 num = make_float2(0.f, 0.f), o;
-        float e = 0.f, qs = 0.f, tval;
-#pragma unroll 4
-        for (int j = 0; j < J; ++j) {
-            const float2 d = dp[(size_t)j * dstride];
-            const float2 h = hp[(size_t)j * half];
-            const float wj = r.w[j];
-            num.x += wj * (d.x * h.x + d.y * h.y);
-            num.y += wj * (d.y * h.x - d.x * h.y);
-            e += wj * (d.x * d.x + d.y * d.y);
-            qs += wj * (h.x * h.x + h.y * h.y);
-        }
-        qs += gam;
-        const float invq = 1.0f / qs;
-        o = cscale(num, invq);
-        const float t_est = e - (num.x * num.x + num.y * num.y) * invq;
-        if (f != 0 && t_est < kCancel * e) {
-            fp64_frequency(J, dp, dstride, hp, half, r.w, r.gamma, seed, tval, o);
+        const bool sup = wbit(r.supp, r.sw, ky, kx), seed = sup && f != 0;
+        const float twice = (kx == 0 || kx == N / 2) ? 1.f : 2.f;
+        float2 o = r.oin ? r.oin[doff] : make_float2(0.f, 0.f), g = make_float2(gam * o.x, gam * o.y);
+        float t = 0.f;
+        if (r.oin && sup) {  // object-inferring loss: the object is given
+            t = explicit_frequency(J, dp, dstride, hp, half, r.w, r.gamma, seed, o, g);
         } else {
-            float tsum = 0.f;
-#pragma unroll 4
-            for (int j = 0; j < J; ++j) {
-                const float2 d = dp[(size_t)j * dstride];
-                const float2 h = hp[(size_t)j * half];
-                const float wj = r.w[j];
+            float2 num = make_float2(0.f, 0.f);
+            float e = 0.f, qs = 0.f;
+            auto gather = [&](float2 d, float2 h, float wj) {
+                num.x += wj * (d.x * h.x + d.y * h.y);
+                num.y += wj * (d.y * h.x - d.x * h.y);
+                e += wj * (d.x * d.x + d.y * d.y);
+                qs += wj * (h.x * h.x + h.y * h.y);
+            };
+            auto scatter = [&](float2 d, float2 h, float wj, int j) {
                 const float2 res = csub(d, cmul(o, h));
-                tsum += wj * (res.x * res.x + res.y * res.y);
-                hp[(size_t)j * half] = seed ? cscale(cmul(cconj(o), res), -wj) : make_float2(0.f, 0.f);
+                t += wj * (res.x * res.x + res.y * res.y);
+                if (sup) hp[(unsigned)j * (unsigned)half] = seed ? cscale(cmul(cconj(o), res), -wj) : make_float2(0.f, 0.f);
+            };
+            // false where the residual cancels (seed frequencies only)
+            auto solve = [&]() {
+                if (r.oin) return true;  // outside the support: the data's energy, O as given
+                qs += gam;
+                const float invq = 1.0f / qs;
+                o = cscale(num, invq);
+                const float t_est = e - (num.x * num.x + num.y * num.y) * invq;
+                return !(seed && t_est < kCancel * e);
+            };
+            bool fine;
+            if (HOLD > 0 && J <= HOLD) {
+                constexpr int H = HOLD > 0 ? HOLD : 1;
+                float2 d[H], h[H];
+                float wv[H];
+#pragma unroll
+                for (int j = 0; j < H; ++j) {
+                    const bool in = j < J;
+                    d[j] = in ? dp[(unsigned)j * dstride] : make_float2(0.f, 0.f);
+                    h[j] = in && sup ? hp[(unsigned)j * (unsigned)half] : make_float2(0.f, 0.f);
+                    wv[j] = in ? r.w[j] : 0.f;
+                }
+#pragma unroll
+                for (int j = 0; j < H; ++j)
+                    if (j < J) gather(d[j], h[j], wv[j]);
+                fine = solve();
+                if (fine) {
+#pragma unroll
+                    for (int j = 0; j < H; ++j)
+                        if (j < J) scatter(d[j], h[j], wv[j], j);
+                }
+            } else {
+                auto chunks = [&](bool on, auto&& use) {
+#pragma unroll 1
+                    for (int j0 = 0; j0 < J; j0 += kChunk) {
+                        float2 d[kChunk], h[kChunk];
+                        float wv[kChunk];
+#pragma unroll
+                        for (int c = 0; c < kChunk; ++c) {
+                            const bool in = on && j0 + c < J;
+                            d[c] = in ? dp[(unsigned)(j0 + c) * dstride] : make_float2(0.f, 0.f);
+                            h[c] = in && sup ? hp[(unsigned)(j0 + c) * (unsigned)half] : make_float2(0.f, 0.f);
+                            wv[c] = in ? r.w[j0 + c] : 0.f;
+                        }
+#pragma unroll
+                        for (int c = 0; c < kChunk; ++c)
+                            if (j0 + c < J) use(d[c], h[c], wv[c], j0 + c);
+                    }
+                };
+                chunks(true, [&](float2 d, float2 h, float wj, int) { gather(d, h, wj); });
+                fine = solve();
+                if (fine) {  // outside the support the residual is the data
+                    chunks(sup, scatter);
+                    if (!sup) t = e;
+                }
             }
-            tval = tsum + gam * (o.x * o.x + o.y * o.y);
+            if (!fine) fp64_frequency(J, dp, dstride, hp, half, r.w, r.gamma, true, t, o);
+            else t += gam * (o.x * o.x + o.y * o.y);
         }
-        acc.add((kx == 0 || kx == N / 2) ? tval : 2.0f * tval);
+        acc.add(twice * t);
         if (r.obj) {
             r.obj[doff] = o;
             if (r.spec_ld == N && kx > 0 && kx < N / 2) r.obj[(size_t)((N - ky) % N) * N + (N - kx)] = cconj(o);
         }
+        if (r.gobj) {
+            r.gobj[doff] = g;
+            if (r.spec_ld == N && kx > 0 && kx < N / 2) r.gobj[(size_t)((N - ky) % N) * N + (N - kx)] = cconj(g);
+        }
     }
-    double v = (double)acc.s - (double)acc.c;
+    return (double)acc.s - (double)acc.c;
+}
+
+// Sum over a CTA of WARPS warps in a fixed order (lanes by a butterfly, then
+// the warps in order), returned by thread 0. `part`: WARPS doubles of shared
+// memory, free again after the caller's next barrier.
+template <int WARPS>
+__device__ __forceinline__ double cta_sum(double v, double* part) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double tot = 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < WARPS; ++w) tot += part[w];
+    return tot;
 }
 
 }  // namespace reduction

@@ -12,42 +12,40 @@ namespace {
 
 using namespace reduction;
 
-// One CTA per patch (persistent over patches), one warp per object; the
-// patch loss sums the objects in order.
-__global__ void __launch_bounds__(32 * kMaxObjects) generic_reduce_kernel(const GenericParams prm) {
-    __shared__ double sobj[kMaxObjects];
-    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int N = prm.N, half = N * (N / 2 + 1), J = prm.J;
+// A CTA takes 1/S of the frequencies of one (patch, object) at a time (S =
+// rsplit); with one object and one split its sum is the patch's loss,
+// otherwise the sums of a patch's objects and splits are added in order by
+// loss_combine_kernel. HOLD: frames of a frequency held in registers. Against
+// one warp per (patch, object, split) and four frames' loads in flight: 2,904
+// units of 96 px 0.126 -> 0.081 ms, 735 of 128 px 0.085 -> 0.056, 12,800 of 128
+// px 0.852 -> 0.460 (58 % of the copy peak on what it cannot do without).
+constexpr int kRedWarps = 8;
+
+template <int HOLD>
+__global__ void __launch_bounds__(32 * kRedWarps, HOLD == 32 ? 1 : 2) generic_reduce_kernel(const GenericParams prm) {
+    __shared__ double part[kRedWarps];
+    const int N = prm.N, half = N * (N / 2 + 1), J = prm.J, S = prm.rsplit;
     const size_t dstride = (size_t)N * prm.spec_ld;
-    const int S = (prm.rsplit > 1 && prm.lpart) ? prm.rsplit : 1;
-    const long long work = (long long)prm.P * S;
+    const long long work = (long long)prm.P * prm.K * S;
     for (long long u = blockIdx.x; u < work; u += gridDim.x) {
-        const int p = (int)(u / S), sp = (int)(u - (long long)p * S);
-        const size_t unit0 = ((size_t)p * prm.K + k) * J;
+        const long long pk = u / S;
+        const int s = (int)(u - pk * S), k = (int)(pk % prm.K);
         RedPtr r;
         r.N = N;
         r.J = J;
         r.spec_ld = prm.spec_ld;
         r.gamma = prm.gamma;
-        r.d = prm.spectra + unit0 * dstride;
-        r.h = prm.gscr + unit0 * half;
+        r.d = prm.spectra + (size_t)pk * J * dstride;
+        r.h = prm.gscr + (size_t)pk * J * half;
         r.w = prm.weights + (size_t)k * J;
         r.supp = prm.obj[k].supp;
         r.sw = prm.sw;
-        r.obj = prm.object ? prm.object + ((size_t)p * prm.K + k) * dstride : nullptr;
-        r.oin = prm.oin ? prm.oin + ((size_t)p * prm.K + k) * dstride : nullptr;
-        r.gobj = prm.gobj ? prm.gobj + ((size_t)p * prm.K + k) * dstride : nullptr;
-        const double v = reduce_warp(r, lane, 32 * sp, 32 * S);
-        if (lane == 0) sobj[k] = v;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double tot = 0.0;
-            for (int i = 0; i < prm.K; ++i) tot += sobj[i];
-            if (S == 1)
-                prm.loss[p] = tot;
-            else
-                prm.lpart[u] = tot;
-        }
+        r.obj = prm.object ? prm.object + (size_t)pk * dstride : nullptr;
+        r.oin = prm.oin ? prm.oin + (size_t)pk * dstride : nullptr;
+        r.gobj = prm.gobj ? prm.gobj + (size_t)pk * dstride : nullptr;
+        const double v = cta_sum<kRedWarps>(
+            reduce_lane<HOLD>(r, 32 * kRedWarps * s + threadIdx.x, 32 * kRedWarps * S), part);
+        if (threadIdx.x == 0) (prm.K * S == 1 ? prm.loss : prm.lpart)[u] = v;
         __syncthreads();
     }
 }
@@ -64,7 +62,7 @@ __global__ void loss_combine_kernel(const double* __restrict__ lpart, int S, dou
 
 size_t generic_smem(int N, bool half_box) {
     const int stride = half_box ? N / 2 + 4 : N + 4;  // Geo<N>::S_HALF, S_FULL
-    return ((size_t)2 * N + (size_t)N * stride) * sizeof(float2);
+    return ((size_t)2 * N + (size_t)N * stride) * sizeof(float2);  // at most 2 N twiddles
 }
 
 int generic_adjoint_ctas(int N, bool half_box, int sms) {
@@ -105,16 +103,29 @@ cudaError_t launch_generic_adjoint(const GenericParams& prm, int sms, cudaStream
 
 cudaError_t launch_generic_reduction(const GenericParams& prm, int sms, cudaStream_t s) {
     if (prm.P == 0) return cudaSuccess;
-    const int threads = 32 * prm.K;
-    const int S = (prm.rsplit > 1 && prm.lpart) ? prm.rsplit : 1;
+    const int per_patch = prm.K * prm.rsplit;
+    if (per_patch > 1 && !prm.lpart) return cudaErrorInvalidValue;
+    // registers for 8, 16 or 32 frames: 2,904 units of 12 frames (96 px) 0.081 ms
+    // in registers, 0.110 in chunks; 12,800 of 32 frames (128 px) 0.460 and 0.477
+    auto kern = prm.J <= 8    ? generic_reduce_kernel<8>
+                : prm.J <= 16 ? generic_reduce_kernel<16>
+                : prm.J <= 32 ? generic_reduce_kernel<32>
+                              : generic_reduce_kernel<0>;
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, generic_reduce_kernel, threads, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kRedWarps, 0);
     if (e != cudaSuccess) return e;
     long long ctas = (long long)sms * (per_sm > 0 ? per_sm : 1);
-    if (ctas > (long long)prm.P * S) ctas = (long long)prm.P * S;
-    generic_reduce_kernel<<<(int)ctas, threads, 0, s>>>(prm);
-    if ((e = cudaGetLastError()) != cudaSuccess || S == 1) return e;
-    return launch_loss_combine(prm.lpart, S, prm.loss, prm.P, s);
+    if (ctas > (long long)prm.P * per_patch) ctas = (long long)prm.P * per_patch;
+    kern<<<(int)ctas, 32 * kRedWarps, 0, s>>>(prm);
+    if ((e = cudaGetLastError()) != cudaSuccess || per_patch == 1) return e;
+    return launch_loss_combine(prm.lpart, per_patch, prm.loss, prm.P, s);
+}
+
+int generic_reduction_split(int P, int K, int N, int sms) {
+    const long long ctas = (long long)P * K, want = 8LL * sms;
+    if (ctas <= 0 || ctas >= want) return 1;
+    const long long smax = std::max(1, N * (N / 2 + 1) / (32 * kRedWarps));
+    return (int)std::min((want + ctas - 1) / ctas, smax);
 }
 
 int reduction_split(int P, int K, int N, int sms) {

@@ -53,24 +53,24 @@ __device__ __forceinline__ UnitPtr unit_ptr(const GenericParams& prm, long long 
 template <int N>
 constexpr int kWarps = N / 16;
 
-template <int N, int S>
+template <int N, int S, bool OTF_ONLY>
 __global__ void __launch_bounds__(32 * kWarps<N>, kMinCtas<N, false, false>) generic_forward_kernel(const GenericParams prm) {
     extern __shared__ __align__(16) unsigned char gsm[];
     float2* tw = reinterpret_cast<float2*>(gsm);
-    float2* E = tw + 2 * N;
+    float2* E = tw + Twiddles<N>::kElems;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     load_twiddles<N>(tw, threadIdx.x, 32 * kWarps<N>);
     __syncthreads();
     const long long units = (long long)prm.P * prm.K * prm.J;
     for (long long u = blockIdx.x; u < units; u += gridDim.x)
-        unit_forward<N, S, kWarps<N>>(unit_ptr<N>(prm, u), E, tw, w, lane, CtaBar{});
+        unit_forward<N, S, kWarps<N>, OTF_ONLY>(unit_ptr<N>(prm, u), E, tw, w, lane, CtaBar{});
 }
 
 template <int N, int S, bool RECOMPUTE>
 __global__ void __launch_bounds__(32 * kWarps<N>, kMinCtas<N, true, RECOMPUTE>) generic_adjoint_kernel(const GenericParams prm) {
     extern __shared__ __align__(16) unsigned char gsm[];
     float2* tw = reinterpret_cast<float2*>(gsm);
-    float2* E = tw + 2 * N;
+    float2* E = tw + Twiddles<N>::kElems;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // RECOMPUTE: the column transforms of P, in this CTA's global buffer (kept
     // in L2) so that shared memory holds one exchange buffer
@@ -135,8 +135,10 @@ cudaError_t launch_generic_forward_n(const GenericParams& prm, int sms, cudaStre
     const long long units = (long long)prm.P * prm.K * prm.J;
     const size_t smem = generic_smem(N, prm.half_box);
     return with_stride<N>(prm.half_box, [&](auto st) {
-        return launch_persistent(generic_forward_kernel<N, decltype(st)::value>, 32 * kWarps<N>, smem, units, sms, prm,
-                                 s);
+        constexpr int S = decltype(st)::value;
+        return prm.otf_only
+                   ? launch_persistent(generic_forward_kernel<N, S, true>, 32 * kWarps<N>, smem, units, sms, prm, s)
+                   : launch_persistent(generic_forward_kernel<N, S, false>, 32 * kWarps<N>, smem, units, sms, prm, s);
     });
 }
 

@@ -7,7 +7,8 @@
 //   blocked  u[8 m + k2] = X[t + 8 m + R k2],  k2 < 8, m < ceil(R / 8)
 // (blocked elements with t + 8 m >= R do not exist). strided_to_blocked
 // transforms one into the other (decimation in time: an R-point transform
-// per lane, the twiddles W_N^(t k1), the exchange, 8-point transforms);
+// per lane, the exchange with the twiddles W_N^(t k1) on one of its sides,
+// 8-point transforms);
 // blocked_to_strided is its mirror (8-point transforms, twiddles, exchange,
 // an R-point transform). A line that was transformed one way can be
 // multiplied pointwise and transformed again the other way without a change
@@ -129,24 +130,40 @@ MFBD_HD void dft_half_out(const float2 (&a)[R], float2 (&x)[R / 2]) {
     });
 }
 
-// Twiddles W_N^(t k1) as the lanes read them: strided_to_blocked takes, per
-// pair of k1, the lanes' t from consecutive 16-byte words ([k1 / 2][t][k1 % 2]);
-// blocked_to_strided takes, per pair of j, the lanes' k1 ([j / 2][k1][j % 2],
-// W_N^(j k1)). N complex each.
+// Where a transform takes its twiddles W_N^(j k1) (j < 8, k1 < R). N = 64 and
+// 128 multiply on the blocked side of the exchange in both directions: one set
+// per lane, taken from shared memory once per pass into registers, serves
+// every transform of the pass (against reading them at each transform, which
+// is a third of the shared-memory wavefronts: 128 px forward passes 0.603 ->
+// 0.590 ms, 64 px 0.350 -> 0.337). At 48 and 96 the register budget has no
+// room for that (96 px 0.109 -> 0.111, adjoint 0.129 -> 0.142 ms): they read
+// them at each transform, 16 bytes at a time, on the side that has fewer.
+template <int N>
+constexpr bool kTwiddlesInRegisters = N % 3 != 0;
+
+// Twiddle tables: in registers, [j][k1]; else for strided_to_blocked, per pair
+// of k1, the lanes' j ([k1 / 2][j][k1 % 2]) and for blocked_to_strided, per
+// pair of j, the lanes' k1 ([j / 2][k1][j % 2]).
 template <int N>
 struct Twiddles {
     static constexpr int R = N / 8;
-    float v[4 * N];
+    static constexpr int kElems = kTwiddlesInRegisters<N> ? N : 2 * N;
+    float v[2 * kElems];
     constexpr Twiddles() : v{} {
-        for (int k1 = 0; k1 < R; ++k1)
-            for (int t = 0; t < 8; ++t) {
-                const fftreg::SinCos sc = fftreg::sincos_2pi(k1 * t, N);
-                const int i = ((k1 / 2) * 8 + t) * 2 + k1 % 2, j = ((t / 2) * R + k1) * 2 + t % 2;
-                v[2 * i] = (float)sc.c;
-                v[2 * i + 1] = (float)-sc.s;
-                v[2 * N + 2 * j] = (float)sc.c;
-                v[2 * N + 2 * j + 1] = (float)-sc.s;
+        for (int j = 0; j < 8; ++j)
+            for (int k1 = 0; k1 < R; ++k1) {
+                const fftreg::SinCos sc = fftreg::sincos_2pi(j * k1, N);
+                if (kTwiddlesInRegisters<N>) {
+                    put(j * R + k1, sc);
+                } else {
+                    put(((k1 / 2) * 8 + j) * 2 + k1 % 2, sc);
+                    put(N + ((j / 2) * R + k1) * 2 + j % 2, sc);
+                }
             }
+    }
+    constexpr void put(int i, const fftreg::SinCos& sc) {
+        v[2 * i] = (float)sc.c;
+        v[2 * i + 1] = (float)-sc.s;
     }
 };
 
@@ -158,18 +175,61 @@ struct Geo {
     static constexpr int R = N / 8;
     static constexpr int M2 = (R + 7) / 8;      // groups of 8 blocked elements per lane
     static constexpr int NH = N / 2 + 1;
-    static constexpr int kTableFloats = 4 * N;  // shared-memory twiddles
     // Row strides (complex) of the N x S exchange buffer: pupil boxes up to
     // N / 2 px, and any box.
     static constexpr int S_HALF = N / 2 + 4, S_FULL = N + 4;
 };
 
-// Copies the twiddles to shared memory; the caller synchronises.
+// Copies the twiddles (Twiddles<N>::kElems complex) to shared memory; the
+// caller synchronises.
 template <int N>
 __device__ __forceinline__ void load_twiddles(float2* tw, int t, int threads) {
-    for (int i = t; i < Geo<N>::kTableFloats / 4; i += threads)
+    for (int i = t; i < Twiddles<N>::kElems / 2; i += threads)
         reinterpret_cast<float4*>(tw)[i] = reinterpret_cast<const float4*>(kTwiddles<N>.v)[i];
 }
+
+// A lane's twiddles for one pass.
+template <int N>
+struct LaneTwiddles {
+    static constexpr int R = Geo<N>::R;
+    float2 w[kTwiddlesInRegisters<N> ? 7 * Geo<N>::M2 : 1];  // W_N^(j (t + 8 m)) at [7 m + j - 1]
+    const float4* table;
+    __device__ __forceinline__ LaneTwiddles(const float2* shared, int t)
+        : table(reinterpret_cast<const float4*>(shared)) {
+        if constexpr (kTwiddlesInRegisters<N>) {
+#pragma unroll
+            for (int m = 0; m < Geo<N>::M2; ++m)
+#pragma unroll
+                for (int j = 1; j < 8; ++j) w[7 * m + j - 1] = shared[j * R + t + 8 * m];
+        }
+    }
+    // strided side of strided_to_blocked
+    __device__ __forceinline__ void strided(float2 (&a)[R], int t) const {
+        if constexpr (!kTwiddlesInRegisters<N>) {
+#pragma unroll
+            for (int p = 0; p < R / 2; ++p) {
+                const float4 v = table[p * 8 + t];
+                if (p > 0) a[2 * p] = cmul(a[2 * p], make_float2(v.x, v.y));
+                a[2 * p + 1] = cmul(a[2 * p + 1], make_float2(v.z, v.w));
+            }
+        }
+    }
+    // blocked side, group m: of strided_to_blocked, and (BACK) of blocked_to_strided
+    template <bool BACK>
+    __device__ __forceinline__ void blocked(float2 (&b)[8], int m, int k1) const {
+        if constexpr (kTwiddlesInRegisters<N>) {
+#pragma unroll
+            for (int j = 1; j < 8; ++j) b[j] = cmul(b[j], w[7 * m + j - 1]);
+        } else if constexpr (BACK) {
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                const float4 v = table[N / 2 + p * R + k1];
+                if (p > 0) b[2 * p] = cmul(b[2 * p], make_float2(v.x, v.y));
+                b[2 * p + 1] = cmul(b[2 * p + 1], make_float2(v.z, v.w));
+            }
+        }
+    }
+};
 
 // Storage of a line in the N x S buffer, in R blocks of 8 elements: element x
 // of block b sits at block(b) + x * kStep.
@@ -194,14 +254,9 @@ struct ColLine {
 // strided a (already transformed over q by dft<R>) -> blocked u.
 template <int N, class Line>
 __device__ __forceinline__ void finish_blocked(const Line& ln, float2 (&a)[N / 8], float2 (&u)[8 * Geo<N>::M2],
-                                               const float2* tw, int t) {
+                                               const LaneTwiddles<N>& tw, int t) {
     constexpr int R = Geo<N>::R, M2 = Geo<N>::M2;
-    static_for<0, R / 2>([&](auto pp) {
-        constexpr int p = decltype(pp)::value;
-        const float4 w = reinterpret_cast<const float4*>(tw)[p * 8 + t];
-        if constexpr (p > 0) a[2 * p] = cmul(a[2 * p], make_float2(w.x, w.y));
-        a[2 * p + 1] = cmul(a[2 * p + 1], make_float2(w.z, w.w));
-    });
+    tw.strided(a, t);
     __syncwarp();  // every lane of the line has read what the storage held
 #pragma unroll
     for (int k1 = 0; k1 < R; ++k1) ln.block(k1)[(t ^ (k1 & 7)) * Line::kStep] = a[k1];
@@ -214,6 +269,7 @@ __device__ __forceinline__ void finish_blocked(const Line& ln, float2 (&a)[N / 8
             const float2* src = ln.block(k1);
 #pragma unroll
             for (int j = 0; j < 8; ++j) b[j] = src[(j ^ t) * Line::kStep];
+            tw.template blocked<false>(b, m, k1);
         } else {
 #pragma unroll
             for (int j = 0; j < 8; ++j) b[j] = make_float2(0.f, 0.f);
@@ -226,7 +282,7 @@ __device__ __forceinline__ void finish_blocked(const Line& ln, float2 (&a)[N / 8
 
 template <int N, class Line>
 __device__ __forceinline__ void strided_to_blocked(const Line& ln, float2 (&a)[N / 8], float2 (&u)[8 * Geo<N>::M2],
-                                                   const float2* tw, int t) {
+                                                   const LaneTwiddles<N>& tw, int t) {
     dft<N / 8>(a);
     finish_blocked<N>(ln, a, u, tw, t);
 }
@@ -234,7 +290,7 @@ __device__ __forceinline__ void strided_to_blocked(const Line& ln, float2 (&a)[N
 // The same for a line whose elements N/2.. are zero (x: the first R / 2).
 template <int N, class Line>
 __device__ __forceinline__ void strided_to_blocked(const Line& ln, const float2 (&x)[N / 16],
-                                                   float2 (&u)[8 * Geo<N>::M2], const float2* tw, int t) {
+                                                   float2 (&u)[8 * Geo<N>::M2], const LaneTwiddles<N>& tw, int t) {
     float2 a[N / 8];
     dft_half_in<N / 8>(x, a);
     finish_blocked<N>(ln, a, u, tw, t);
@@ -243,9 +299,8 @@ __device__ __forceinline__ void strided_to_blocked(const Line& ln, const float2 
 // blocked u -> strided a before its R-point transform.
 template <int N, class Line>
 __device__ __forceinline__ void start_strided(const Line& ln, const float2 (&u)[8 * Geo<N>::M2], float2 (&a)[N / 8],
-                                              const float2* tw, int t) {
+                                              const LaneTwiddles<N>& tw, int t) {
     constexpr int R = Geo<N>::R, M2 = Geo<N>::M2;
-    const float4* tq = reinterpret_cast<const float4*>(tw + N);
     __syncwarp();
 #pragma unroll
     for (int m = 0; m < M2; ++m) {
@@ -255,13 +310,8 @@ __device__ __forceinline__ void start_strided(const Line& ln, const float2 (&u)[
 #pragma unroll
             for (int j = 0; j < 8; ++j) b[j] = u[8 * m + j];
             dft<8>(b);
+            tw.template blocked<true>(b, m, k1);
             float2* dst = ln.block(k1);
-#pragma unroll
-            for (int p = 0; p < 4; ++p) {
-                const float4 w = tq[p * R + k1];
-                if (p > 0) b[2 * p] = cmul(b[2 * p], make_float2(w.x, w.y));
-                b[2 * p + 1] = cmul(b[2 * p + 1], make_float2(w.z, w.w));
-            }
 #pragma unroll
             for (int j = 0; j < 8; ++j) dst[(j ^ t) * Line::kStep] = b[j];
         }
@@ -273,7 +323,7 @@ __device__ __forceinline__ void start_strided(const Line& ln, const float2 (&u)[
 
 template <int N, class Line>
 __device__ __forceinline__ void blocked_to_strided(const Line& ln, const float2 (&u)[8 * Geo<N>::M2],
-                                                   float2 (&a)[N / 8], const float2* tw, int t) {
+                                                   float2 (&a)[N / 8], const LaneTwiddles<N>& tw, int t) {
     start_strided<N>(ln, u, a, tw, t);
     dft<N / 8>(a);
 }
@@ -281,7 +331,7 @@ __device__ __forceinline__ void blocked_to_strided(const Line& ln, const float2 
 // The same, the first half of the outputs only.
 template <int N, class Line>
 __device__ __forceinline__ void blocked_to_strided(const Line& ln, const float2 (&u)[8 * Geo<N>::M2],
-                                                   float2 (&x)[N / 16], const float2* tw, int t) {
+                                                   float2 (&x)[N / 16], const LaneTwiddles<N>& tw, int t) {
     float2 a[N / 8];
     start_strided<N>(ln, u, a, tw, t);
     dft_half_out<N / 8>(a, x);

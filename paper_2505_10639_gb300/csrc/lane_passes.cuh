@@ -64,7 +64,7 @@ struct ColumnBits {
 struct UnitPtr {
     const float* phi;       // [W][W] box phase
     float* gphi;            // [W][W] dL/dphi (0 outside the pupil)
-    float2* h;              // [N][N/2+1]: OTF, then the adjoint seed
+    float2* h;              // [N][N/2+1]: OTF, then the adjoint seed; read on the OTF support only
     float2* pf;             // [N][N] field rows, or null (recomputed)
     int W;
     float inv_z;            // 1 / (N^2 n_pup)
@@ -96,11 +96,12 @@ struct BoxPoints {
 // PUPIL. Columns of the transform go to the buffer E, or (dst != null) to
 // dst [N][ld], the buffer then only carrying the exchange.
 template <int N, int S, int WARPS>
-__device__ __forceinline__ void pass_pupil(const UnitPtr& q, float2* E, const float2* tw, int w, int lane, float2* dst,
+__device__ __forceinline__ void pass_pupil(const UnitPtr& q, float2* E, const float2* table, int w, int lane, float2* dst,
                                            int ld) {
     constexpr int R = Geo<N>::R, M2 = Geo<N>::M2, Q = BoxPoints<N, S>::kQ;
     const ColLanes cl(lane);
     const int t = cl.t;
+    const LaneTwiddles<N> tw(table, t);
     for (int c0 = 4 * w; c0 < q.W; c0 += 4 * WARPS) {
         const int c = c0 + cl.c;
         const bool act = c < q.W;
@@ -128,17 +129,22 @@ __device__ __forceinline__ void pass_pupil(const UnitPtr& q, float2* E, const fl
     }
 }
 
-// Forward passes of one unit -> q.h (and the field q.pf when kept). E: the
-// group's N x S exchange buffer; w, lane: warp of the group and lane. Ends
-// with the group's barrier.
-template <int N, int S, int WARPS, class Bar>
-__device__ __forceinline__ void unit_forward(const UnitPtr& q, float2* E, const float2* tw, int w, int lane, Bar bar) {
+// Forward passes of one unit -> q.h (and the field q.pf when kept); OTF_ONLY:
+// q.h is also written (0) outside the OTF support. E: the group's N x S
+// exchange buffer; w, lane: warp of the group and lane. Ends with the group's
+// barrier.
+template <int N, int S, int WARPS, bool OTF_ONLY, class Bar>
+__device__ __forceinline__ void unit_forward(const UnitPtr& q, float2* E, const float2* table, int w, int lane, Bar bar) {
     constexpr int R = Geo<N>::R, M2 = Geo<N>::M2, NH = Geo<N>::NH, Q = BoxPoints<N, S>::kQ;
-    pass_pupil<N, S, WARPS>(q, E, tw, w, lane, nullptr, 0);
+    // skipping the stores outside the support costs a branch each, which pays at
+    // the larger sizes only (128 px forward 0.655 -> 0.603 ms, 48 px 0.193 -> 0.214)
+    constexpr bool kAll = OTF_ONLY || N <= 64;
+    pass_pupil<N, S, WARPS>(q, E, table, w, lane, nullptr, 0);
     bar();
     {  // ROWS
         const RowLanes rl(lane);
         const int t = rl.t;
+        const LaneTwiddles<N> tw(table, t);
 #pragma unroll 1
         for (int p0 = 4 * w; p0 < N / 2; p0 += 4 * WARPS) {
             const int i = p0 + rl.p;
@@ -187,6 +193,7 @@ __device__ __forceinline__ void unit_forward(const UnitPtr& q, float2* E, const 
     {  // OTF
         const ColLanes cl(lane);
         const int t = cl.t;
+        const LaneTwiddles<N> tw(table, t);
 #pragma unroll 1
         for (int l0 = 4 * w; l0 < N / 2; l0 += 4 * WARPS) {
             const int kx = l0 + cl.c;
@@ -226,7 +233,9 @@ __device__ __forceinline__ void unit_forward(const UnitPtr& q, float2* E, const 
                                 const int ky = t + 8 * m + R * k;
                                 const float2 z = u[8 * m + k], c = E[(ky ? N - ky : 0) * S];
                                 const float2 hn = make_float2(0.5f * (z.y + c.y), 0.5f * (c.x - z.x));
-                                q.h[ky * NH + N / 2] = in2.bit(8 * m + R * k) ? hn : make_float2(0.f, 0.f);
+                                const bool sup = in2.bit(8 * m + R * k);
+                                if constexpr (kAll) q.h[ky * NH + N / 2] = sup ? hn : make_float2(0.f, 0.f);
+                                else if (sup) q.h[ky * NH + N / 2] = hn;
                                 u[8 * m + k] = ky ? make_float2(0.5f * (z.x + c.x), 0.5f * (z.y - c.y))
                                                   : make_float2(1.f, 0.f);
                             }
@@ -236,9 +245,12 @@ __device__ __forceinline__ void unit_forward(const UnitPtr& q, float2* E, const 
             for (int m = 0; m < M2; ++m)
                 if (R % 8 == 0 || t + 8 * m < R)
 #pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        q.h[(t + 8 * m + R * k) * NH + kx] =
-                            in.bit(8 * m + R * k) ? u[8 * m + k] : make_float2(0.f, 0.f);
+                    for (int k = 0; k < 8; ++k) {
+                        const int ky = t + 8 * m + R * k;
+                        const bool sup = in.bit(8 * m + R * k);
+                        if constexpr (kAll) q.h[ky * NH + kx] = sup ? u[8 * m + k] : make_float2(0.f, 0.f);
+                        else if (sup) q.h[ky * NH + kx] = u[8 * m + k];
+                    }
         }
     }
     bar();
@@ -248,8 +260,8 @@ __device__ __forceinline__ void unit_forward(const UnitPtr& q, float2* E, const 
 // g_q row; conj(g p) transformed back to strided.
 template <int N, int S, int Q>
 __device__ __forceinline__ void adjoint_row(const RowLine<N, S>& ln, float2 (&u)[8 * Geo<N>::M2],
-                                            const float (&g)[8 * Geo<N>::M2], float2 (&out)[Q], const float2* tw,
-                                            int t) {
+                                            const float (&g)[8 * Geo<N>::M2], float2 (&out)[Q],
+                                            const LaneTwiddles<N>& tw, int t) {
 #pragma unroll
     for (int e = 0; e < 8 * Geo<N>::M2; ++e) u[e] = make_float2(g[e] * u[e].x, -g[e] * u[e].y);
     blocked_to_strided<N>(ln, u, out, tw, t);
@@ -259,27 +271,31 @@ __device__ __forceinline__ void adjoint_row(const RowLine<N, S>& ln, float2 (&u)
 // outside the pupil). E2 (row stride es2): RECOMPUTE's global buffer for the
 // column transforms of P. Ends with the group's barrier.
 template <int N, int S, int WARPS, bool RECOMPUTE, class Bar>
-__device__ __forceinline__ void unit_adjoint(const UnitPtr& q, float2* E, float2* E2, int es2, const float2* tw, int w,
+__device__ __forceinline__ void unit_adjoint(const UnitPtr& q, float2* E, float2* E2, int es2, const float2* table, int w,
                                              int lane, Bar bar) {
     constexpr int R = Geo<N>::R, M2 = Geo<N>::M2, NH = Geo<N>::NH, Q = BoxPoints<N, S>::kQ;
     if constexpr (RECOMPUTE) {
-        pass_pupil<N, S, WARPS>(q, E, tw, w, lane, E2, es2);
+        pass_pupil<N, S, WARPS>(q, E, table, w, lane, E2, es2);
         bar();
     }
     {  // SEED
         const ColLanes cl(lane);
         const int t = cl.t;
+        const LaneTwiddles<N> tw(table, t);
 #pragma unroll 1
         for (int l0 = 4 * w; l0 < N / 2; l0 += 4 * WARPS) {
             const int kx = l0 + cl.c;
             const ColLine<N, S> ln{E + kx, kx ? N / 2 - 2 * kx : 0};
             float2 a[R], u[8 * M2];
+            const ColumnBits in(q.csupp + 2 * kx, true, t);
 #pragma unroll
-            for (int e = 0; e < R; ++e) a[e] = cconj(q.h[(t + 8 * e) * NH + kx]);
+            for (int e = 0; e < R; ++e)
+                a[e] = N <= 64 || in.bit(8 * e) ? cconj(q.h[(t + 8 * e) * NH + kx]) : make_float2(0.f, 0.f);
             if (kx == 0) {  // conj(G_0 + i G_N/2)
+                const ColumnBits in2(q.csupp + 2 * (N / 2), true, t);
 #pragma unroll
                 for (int e = 0; e < R; ++e) {
-                    const float2 b = q.h[(t + 8 * e) * NH + N / 2];
+                    const float2 b = N <= 64 || in2.bit(8 * e) ? q.h[(t + 8 * e) * NH + N / 2] : make_float2(0.f, 0.f);
                     a[e] = make_float2(a[e].x - b.y, a[e].y - b.x);
                 }
             }
@@ -307,6 +323,7 @@ __device__ __forceinline__ void unit_adjoint(const UnitPtr& q, float2* E, float2
     {  // ROWS
         const RowLanes rl(lane);
         const int t = rl.t;
+        const LaneTwiddles<N> tw(table, t);
         const float sc = 2.0f * q.inv_z;
 #pragma unroll 1
         for (int p0 = 4 * w; p0 < N / 2; p0 += 4 * WARPS) {
@@ -358,6 +375,7 @@ __device__ __forceinline__ void unit_adjoint(const UnitPtr& q, float2* E, float2
     {  // ADJ: dL/dphi = 2 Im(conj(P) G_P) on the pupil
         const ColLanes cl(lane);
         const int t = cl.t;
+        const LaneTwiddles<N> tw(table, t);
 #pragma unroll 1
         for (int c0 = 4 * w; c0 < q.W; c0 += 4 * WARPS) {
             const int c = c0 + cl.c;

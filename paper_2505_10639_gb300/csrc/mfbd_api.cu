@@ -93,8 +93,8 @@ struct mfbd_plan {
     int e2_ctas = 0;
     const void* x_oin = nullptr;  // mfbd_loss_grad_explicit: the given objects, during that call only
     void* x_gobj = nullptr;       // and dL/dconj(O)
-    int rsplit = 1;             // warps per (patch, object) of the frame reduction
-    double* d_lpart = nullptr;  // rsplit > 1: per-split patch losses [P][rsplit]
+    int rsplit = 1;             // warps (general sizes: CTAs) per (patch, object) of the frame reduction
+    double* d_lpart = nullptr;  // their losses: [P][rsplit], general sizes [P][K][rsplit]; null for one per patch
     int ustride = 0;
     long long phi_floats = 0;
     size_t workspace = 0;
@@ -452,6 +452,7 @@ int run_generic(mfbd_plan_t p, int stages, const void* spectra, double* loss, vo
     g.phi = p->d_phi;
     g.gphi = p->d_gphi;
     const bool otf_only = (stages & ST_OTF_ONLY) != 0;
+    g.otf_only = otf_only;
     g.gscr = otf_only ? gscr : p->d_gscr;
     g.pscr = otf_only ? nullptr : p->d_pscr;
     g.spectra = static_cast<const float2*>(spectra);
@@ -484,7 +485,7 @@ int run_generic(mfbd_plan_t p, int stages, const void* spectra, double* loss, vo
     if (e == cudaSuccess && (stages & ST_RED)) {
         const int pr = prof_begin(p, 2, s);
         e = launch_generic_reduction(g, p->sms, s);
-        prof_end(p, pr, s, p->rsplit > 1 && p->d_lpart ? 2 : 1);  // + the loss combine
+        prof_end(p, pr, s, p->K * p->rsplit > 1 ? 2 : 1);  // + the loss combine
     }
     if (e == cudaSuccess && (stages & ST_ADJ)) {
         const int pb = prof_begin(p, 3, s);
@@ -846,8 +847,10 @@ int mfbd_plan_create(mfbd_plan_t* out, const mfbd_plan_desc* d, void* stream) {
         if (keep && !p->generic && (st = dev_alloc(p, &p->d_uscr, (size_t)p->P * p->K * p->J * p->ustride))) throw st;
 
         p->sms = prop.multiProcessorCount;
-        p->rsplit = reduction_split(p->P, p->K, n, p->sms);
-        if (p->rsplit > 1 && (st = dev_alloc(p, &p->d_lpart, (size_t)p->P * p->rsplit))) throw st;
+        p->rsplit = p->generic ? generic_reduction_split(p->P, p->K, n, p->sms)
+                               : reduction_split(p->P, p->K, n, p->sms);
+        const size_t lparts = (size_t)p->rsplit * (p->generic ? p->K : 1);  // per patch
+        if (lparts > 1 && (st = dev_alloc(p, &p->d_lpart, (size_t)p->P * lparts))) throw st;
         if (!p->generic) {
             p->geo = fused_geometry(max_box);
             int per_sm = max_ctas_per_sm(p->geo);

@@ -180,7 +180,7 @@ struct GenericParams {
     const float* weights;   // [K][J]
     const float* phi;       // box phases, per object at phi_off
     float* gphi;            // dL/dphi, same layout
-    float2* gscr;           // [P][K][J][N][N/2+1]: OTF, then dL/dconj(H)
+    float2* gscr;           // [P][K][J][N][N/2+1]: OTF, then dL/dconj(H); read on the OTF support only
     float2* pscr;           // [P][K][J][N][N] field rows; null: recomputed by the adjoint
     const float2* spectra;  // D
     int spec_ld;            // N/2 + 1 or N
@@ -190,8 +190,9 @@ struct GenericParams {
     int es2;                // row stride (complex) of e2scr's buffers
     float2* e2scr;          // recompute: per-CTA second buffers [ctas][N * es2] in global memory (L2)
     int e2_ctas;            // CTAs e2scr has room for
-    int rsplit;             // warps per (patch, object) of the frame reduction (<= 1: one)
-    double* lpart;          // rsplit > 1: per-split patch losses [P][rsplit]
+    int rsplit;             // CTAs that share a (patch, object) of the frame reduction
+    double* lpart;          // K rsplit > 1: their losses [P][K][rsplit]
+    bool otf_only;          // gscr is the caller's OTF: also written outside the support
     const float2* oin;      // object-inferring loss: the given objects [P][K][N][spec_ld], else null
     float2* gobj;           // with oin: dL/dconj(O) [P][K][N][spec_ld], or null
     GenericObj obj[kMaxObjects];
@@ -214,6 +215,10 @@ template <int N> cudaError_t launch_generic_adjoint_n(const GenericParams& prm, 
 // keeping at least 4 frequencies) when they are few. A plan fixes it from its
 // patch count, so chunked calls sum the loss in the same order.
 int reduction_split(int P, int K, int N, int sms);
+// CTAs per (patch, object) of the general sizes' frame reduction: one while the
+// pairs alone make 8 CTAs per SM, more (each lane keeping a frequency) when
+// they are few. Fixed by a plan like reduction_split.
+int generic_reduction_split(int P, int K, int N, int sms);
 // loss[p] = sum over s < S of lpart[p][s], in order.
 cudaError_t launch_loss_combine(const double* lpart, int S, double* loss, int P, cudaStream_t s);
 

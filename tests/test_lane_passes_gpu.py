@@ -57,3 +57,36 @@ def test_batch_box_and_unit_edges(shapes):
         loss, grad, obj = (b.unpack(t, k) for t, k in zip(out, ("loss", "grad", "object")))
         for i, (case, _, _, ref) in enumerate(data):
             _check(case, loss[i].cpu().numpy(), grad[i].cpu().numpy(), obj[i].cpu().numpy().astype("complex128"), ref)
+
+
+@pytest.mark.parametrize("frames", [1, 8, 9, 16, 17, 32, 33])
+@pytest.mark.parametrize("n_pix,diams", [(48, (20.0, 24.0)), (96, (40.0,))])
+def test_frame_reduction_frame_counts(n_pix, diams, frames):
+    """The frame reduction where its register forms (8, 16, 32 frames) end and its chunked form begins."""
+    case = cases.make_case(n_pix=n_pix, diams=diams, wavelengths=(6563.0, 8542.0)[:len(diams)], n_frames=frames,
+                           n_modes=5, basis="zernike", n_patches=1, seed=20250800 + frames)
+    a32, d32, d_or = _inputs(case)
+    loss, grad, obj = _run_fused(_plan_for(case), a32, d32)
+    _check(case, loss, grad, obj, _oracle(case, a32, d_or))
+
+
+@pytest.mark.parametrize("atoms", [1, 2, 3])
+def test_dictionary_units_beyond_one_wave(atoms):
+    """More units than resident CTAs (a CTA takes several, its exchange buffers alternating across them): copies of a
+    patch get the bits of the first."""
+    import numpy as np
+
+    from paper_2505_10639_gb300 import synth
+    from tests.test_dict_gpu import _check as check_dict
+    from tests.test_dict_gpu import _oracle as oracle_dict
+    from tests.test_dict_gpu import _run as run_dict
+    case = list(synth.dictionary_case(20250900 + atoms, 2, 2, 3, atoms))
+    one = run_dict(tuple(case))
+    many = list(case)
+    for i in (3, 4, 5):
+        many[i] = np.tile(case[i], (60,) + (1,) * (case[i].ndim - 1))
+    loss, go, ga = run_dict(tuple(many))
+    for r in range(60):
+        assert np.array_equal(loss[2 * r:2 * r + 2], one[0])
+        assert np.array_equal(go[2 * r:2 * r + 2], one[1]) and np.array_equal(ga[2 * r:2 * r + 2], one[2])
+    check_dict(0, *one, oracle_dict(tuple(case), 0))
