@@ -7,26 +7,30 @@
 // g_ikj = Re F^H[conj(Phi_i) (-2 gamma_kj R_kj)] (F^H unnormalised):
 //   dL/da_ikj = o_k g_ikj,  dL/do_k = sum_j sum_i a_ikj g_ikj.
 //
-// dict_unit_kernel: one warp per unit (patch, object, frame), N = 64.
-//   Forward, per atom i: lane y forms rows y and y + N/2 of o a_i as one
-//   complex line (16-byte loads), transforms it and splits it into the two
-//   rows' half spectra (the real columns 0 and N/2 stored packed as one
-//   complex column); lane kx transforms half-spectrum column kx (lane 0 the
-//   packed column, which it leaves in shared memory for all lanes to split,
-//   two rows each) and accumulates X_i Phi_i into the unit's model spectrum
-//   in shared memory. Then the residual, the unit's loss (FP64 sums of FP32
-//   terms; columns 0 and N/2 once, the others twice) and G = -2 gamma R in
-//   place of the model.
+// dict_unit_kernel: one CTA of eight warps per unit (patch, object, frame),
+// N = 64, persistent; lines of eight lanes (lane8.cuh), every warp holding the
+// same four row pairs and four half-spectrum columns of every atom.
+//   Forward, per atom i: rows y and y + N/2 of o a_i as one complex line,
+//   transformed; then the half-spectrum columns (the two rows' spectra split
+//   on load, columns 0 and N/2 packed in line 0), transformed, times Phi_i,
+//   accumulated in registers: a lane owns eight frequencies of one column.
+//   Then the residual, the unit's loss (FP64 sums of FP32 terms; columns 0 and
+//   N/2 once, the others twice) and conj(G) = -2 gamma conj(R) in place.
 //   Backward, per atom i: the inverse of the half spectrum conj(Phi_i) G
-//   (columns along ky, 0 and N/2 packed, then Hermitian-extended row pairs,
-//   as the mosaic's object images) gives rows y and y + N/2 of g_i in lane
-//   y: dL/da_i = o g_i is stored (16-byte stores), and a_i g_i accumulated
-//   into the unit's share of dL/do in shared memory, written out at the end.
+//   (columns along ky, then the packed row pairs) gives g_i; dL/da_i = o g_i
+//   is stored and a_i g_i accumulated in registers into the unit's share of
+//   dL/do, written out at the end.
+// The atoms alternate between two exchange buffers, so that one CTA barrier
+// per atom (rows to columns, or back) is enough.
+//   HBM is the floor (coefficient maps in and their gradient out); the L1 data
+//   path bounds it (shared-memory exchanges, atom transforms: 65 % of its
+//   wavefronts, issue 32 %). 5,400 units of 8 atoms: 2.63 ms with one warp per
+//   unit (a 64-point line per lane, 4 warps an SM), 0.936 ms with this.
 // dict_combine_kernel: dL/do_k = the units' shares summed over frames in
 // frame order; the patch loss = the units' losses summed over (k, j) in order.
 #include "../../include/mfbd.h"
 #include "mfbd_internal.h"
-#include "line_fft.cuh"
+#include "lane_passes.cuh"
 
 #include <cuda_runtime.h>
 
@@ -36,14 +40,13 @@ using namespace mfbd_dev;
 
 namespace {
 
-using namespace mfbd_dev::linefft;
+using namespace mfbd_dev::lanepass;
 
-constexpr int kDN = 64, kDNH = kDN / 2 + 1, kDES = kDNH;  // exchange stride 33 (odd)
-constexpr int kDoLd = kDN + 1;                             // dL/do rows, padded
-// shared memory of one unit: exchange buffer, model / G spectrum, dL/do share,
-// lane 0's packed column
-constexpr size_t kDictSmem = 2 * (size_t)kDN * kDES * sizeof(float2) + (size_t)kDN * kDoLd * sizeof(float) +
-                             (size_t)kDN * sizeof(float2);
+constexpr int kDN = 64, kDNH = kDN / 2 + 1;
+constexpr int kDS = Geo<kDN>::S_HALF;  // row stride of an exchange buffer
+constexpr int kDWarps = 8;             // one group of four lines each, in every pass
+// shared memory of a CTA: the twiddles and two exchange buffers
+constexpr size_t kDictSmem = ((size_t)kDN + 2 * (size_t)kDN * kDS) * sizeof(float2);
 
 struct DictParams {
     int P, K, J, M;
@@ -57,35 +60,29 @@ struct DictParams {
     double* unit_loss;       // [P][K][J] (workspace)
 };
 
-// rows y and y + N/2 of o a (a = 0: o alone is not needed) as one complex line
-__device__ __forceinline__ void load_product_rows(const float* o, const float* a, int y, float2 (&v)[kDN]) {
-    const float4* o0 = reinterpret_cast<const float4*>(o + y * kDN);
-    const float4* o1 = reinterpret_cast<const float4*>(o + (y + kDN / 2) * kDN);
-    const float4* a0 = reinterpret_cast<const float4*>(a + y * kDN);
-    const float4* a1 = reinterpret_cast<const float4*>(a + (y + kDN / 2) * kDN);
-#pragma unroll
-    for (int c = 0; c < kDN / 4; ++c) {
-        const float4 p = o0[c], q = o1[c], s = a0[c], t = a1[c];
-        v[4 * c] = make_float2(p.x * s.x, q.x * t.x);
-        v[4 * c + 1] = make_float2(p.y * s.y, q.y * t.y);
-        v[4 * c + 2] = make_float2(p.z * s.z, q.z * t.z);
-        v[4 * c + 3] = make_float2(p.w * s.w, q.w * t.w);
-    }
-}
-
 }  // namespace
 
 namespace {
 
-__global__ void __launch_bounds__(32) dict_unit_kernel(const DictParams prm) {
+__global__ void __launch_bounds__(32 * kDWarps, 2) dict_unit_kernel(const DictParams prm) {
     extern __shared__ __align__(16) unsigned char dsm[];
-    float2* E = reinterpret_cast<float2*>(dsm);             // [N][33] exchange
-    float2* A = E + kDN * kDES;                               // [N][33] model spectrum, then G
-    float* DO = reinterpret_cast<float*>(A + kDN * kDES);     // [N][65] the unit's share of dL/do
-    float2* Z = reinterpret_cast<float2*>(DO + kDN * kDoLd);  // [N] a packed column
-    const int lane = threadIdx.x;
+    float2* table = reinterpret_cast<float2*>(dsm);
+    float2* const buf0 = table + kDN;
+    __shared__ double part[kDWarps];
+    __shared__ float2 snyq[kDN];  // column N/2, each element private to a lane of line 0
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    load_twiddles<kDN>(table, threadIdx.x, 32 * kDWarps);
+    __syncthreads();
     const long long units = (long long)prm.P * prm.K * prm.J;
     const bool backward = prm.grad_coeff != nullptr || prm.unit_gobj != nullptr;
+    // this lane's four-line group: the row pair (i, i + 32) and the column kx;
+    // at 64 points a blocked line holds the same elements t + 8 e as a strided one
+    const RowLanes rl(lane);
+    const ColLanes cl(lane);
+    const int i = 4 * w + rl.p, tr = rl.t, kx = 4 * w + cl.c, tc = cl.t;
+    const int shift = kx ? kDN / 2 - 2 * kx : 0;
+    const int r0 = i * kDN + tr, r1 = (i + kDN / 2) * kDN + tr;  // first element of the rows' lines
+    int b = 0;  // exchange buffer of the next atom: one barrier per atom and pass pair
     for (long long u = blockIdx.x; u < units; u += gridDim.x) {
         const int j = (int)(u % prm.J);
         const long long pk = u / prm.J;
@@ -94,169 +91,179 @@ __global__ void __launch_bounds__(32) dict_unit_kernel(const DictParams prm) {
         const float* a = prm.coeff + (size_t)u * prm.M * kDN * kDN;
         const float2* I = prm.spectra + (size_t)u * kDN * kDNH;
         const float gam = prm.gamma[k * prm.J + j];
-        for (int e = lane; e < kDN * kDES; e += 32) A[e] = make_float2(0.f, 0.f);
-        __syncwarp();
         // ------------------------------------------- model: sum_i F(o a_i) Phi_i
-        for (int i = 0; i < prm.M; ++i) {
-            const float2* Phi = prm.atom_otf + (size_t)i * kDN * kDNH;
-            float2 v[kDN];
-            load_product_rows(o, a + (size_t)i * kDN * kDN, lane, v);
-            line_fft<kDN, -1>(v, 0);
-            // rows y, y + N/2: their half spectra; columns 0 and N/2 packed in column 0
-            E[lane * kDES] = make_float2(v[0].x, v[kDN / 2].x);
-            E[(lane + kDN / 2) * kDES] = make_float2(v[0].y, v[kDN / 2].y);
-            fftreg::static_for<1, kDN / 2>([&](auto kk) {
-                constexpr int kq = decltype(kk)::value;
-                const float2 pc = conj_partner<kDN, kq>(v);
-                const float2 ra = cscale(cadd(v[kq], pc), 0.5f);
-                const float2 d = cscale(csub(v[kq], pc), 0.5f);
-                E[lane * kDES + kq] = ra;
-                E[(lane + kDN / 2) * kDES + kq] = make_float2(d.y, -d.x);
-            });
-            __syncwarp();
+        float2 mod[8];  // column kx
+        float2* const nyq = snyq + tc;  // and, in the lanes of line 0, column N/2
 #pragma unroll
-            for (int ky = 0; ky < kDN; ++ky) v[ky] = E[ky * kDES + lane];
-            __syncwarp();
-            line_fft<kDN, -1>(v, 0);
-            // lanes 1 .. 31 accumulate their column; lane 0 leaves the packed one
+        for (int e = 0; e < 8; ++e) mod[e] = make_float2(0.f, 0.f);
+        if (kx == 0) {
 #pragma unroll
-            for (int ky = 0; ky < kDN; ++ky) {
-                const float2 ph = Phi[ky * kDNH + lane];
-                if (lane > 0) {
-                    float2* acc = &A[ky * kDES + lane];
-                    *acc = cadd(*acc, cmul(v[ky], ph));
-                } else {
-                    Z[ky] = v[ky];
+            for (int e = 0; e < 8; ++e) nyq[8 * e] = make_float2(0.f, 0.f);
+        }
+        float o0[8], o1[8], a0[8], a1[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            o0[e] = o[r0 + 8 * e];
+            o1[e] = o[r1 + 8 * e];
+            a0[e] = a[r0 + 8 * e];
+            a1[e] = a[r1 + 8 * e];
+        }
+        for (int m = 0; m < prm.M; ++m) {
+            float2* E = buf0 + b * (kDN * kDS);
+            b ^= 1;
+            {
+                const RowLine<kDN, kDS> ln{E + i * kDS};
+                float2 v[8], z[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = make_float2(o0[e] * a0[e], o1[e] * a1[e]);
+                if (m + 1 < prm.M) {  // the next atom's maps arrive under this atom's transforms
+                    const float* an = a + (size_t)(m + 1) * kDN * kDN;
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        a0[e] = an[r0 + 8 * e];
+                        a1[e] = an[r1 + 8 * e];
+                    }
+                }
+                strided_to_blocked<kDN>(ln, v, z, LaneTwiddles<kDN>(table, tr), tr);
+                __syncwarp();
+#pragma unroll
+                for (int e = 0; e < 8; ++e) ln.block(e)[tr] = z[e];
+            }
+            __syncthreads();
+            const float2* Phi = prm.atom_otf + (size_t)m * kDN * kDNH;
+            const ColLine<kDN, kDS> ln{E + kx, shift};
+            float2 v[8], x[8];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {  // the two rows' half spectra at kx; line 0: columns 0 and N/2 packed
+                const float2 p = ln.block(e)[tc * kDS], q = ln.block(e + 4)[tc * kDS];
+                v[e] = kx ? make_float2(0.5f * (p.x + q.x), 0.5f * (p.y - q.y)) : make_float2(p.x, q.x);
+                v[e + 4] = kx ? make_float2(0.5f * (p.y + q.y), 0.5f * (q.x - p.x)) : make_float2(p.y, q.y);
+            }
+            strided_to_blocked<kDN>(ln, v, x, LaneTwiddles<kDN>(table, tc), tc);
+            if (w == 0) {  // the warp of line 0 splits its packed columns through the line's storage
+                __syncwarp();
+                if (kx == 0) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) E[(tc + 8 * e) * kDS] = x[e];
+                }
+                __syncwarp();
+                if (kx == 0) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int ky = tc + 8 * e;
+                        const float2 z = x[e], c = E[((kDN - ky) & (kDN - 1)) * kDS];
+                        const float2 h = make_float2(0.5f * (z.y + c.y), 0.5f * (c.x - z.x));
+                        nyq[8 * e] = cadd(nyq[8 * e], cmul(h, Phi[ky * kDNH + kDN / 2]));
+                        x[e] = make_float2(0.5f * (z.x + c.x), 0.5f * (z.y - c.y));
+                    }
                 }
             }
-            __syncwarp();
-            // X(ky, 0) = (Z[ky] + conj Z[-ky]) / 2, X(ky, N/2) = (Z[ky] - conj Z[-ky]) / (2i)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int ky = lane + h * (kDN / 2);
-                const float2 z = Z[ky], zp = cconj(Z[(kDN - ky) & (kDN - 1)]);
-                const float2 x0 = cscale(cadd(z, zp), 0.5f);
-                const float2 d = cscale(csub(z, zp), 0.5f);
-                const float2 xh = make_float2(d.y, -d.x);
-                A[ky * kDES] = cadd(A[ky * kDES], cmul(x0, Phi[ky * kDNH]));
-                A[ky * kDES + kDN / 2] = cadd(A[ky * kDES + kDN / 2], cmul(xh, Phi[ky * kDNH + kDN / 2]));
-            }
-            __syncwarp();
+            for (int e = 0; e < 8; ++e) mod[e] = cadd(mod[e], cmul(x[e], Phi[(tc + 8 * e) * kDNH + kx]));
         }
-        // --------------------------------- residual, loss, G = -2 gamma R in A
+        // --------------------- residual, loss, conj(G) = -2 gamma conj(R) in place
         double lacc = 0.0;
-        if (lane > 0) {
-#pragma unroll 8
-            for (int ky = 0; ky < kDN; ++ky) {
-                const float2 d = I[ky * kDNH + lane], m = A[ky * kDES + lane];
-                const float2 r = make_float2(d.x - m.x, d.y - m.y);
-                lacc += 2.0 * (double)(r.x * r.x + r.y * r.y);
-                A[ky * kDES + lane] = cscale(r, -2.f * gam);
-            }
-        }
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int ky = lane + h * (kDN / 2);
-#pragma unroll
-            for (int c = 0; c <= kDN / 2; c += kDN / 2) {
-                const float2 d = I[ky * kDNH + c], m = A[ky * kDES + c];
-                const float2 r = make_float2(d.x - m.x, d.y - m.y);
-                lacc += (double)(r.x * r.x + r.y * r.y);
-                A[ky * kDES + c] = cscale(r, -2.f * gam);
+        for (int e = 0; e < 8; ++e) {
+            const float2 d = I[(tc + 8 * e) * kDNH + kx];
+            const float2 r = make_float2(d.x - mod[e].x, d.y - mod[e].y);
+            lacc += (kx ? 2.0 : 1.0) * (double)(r.x * r.x + r.y * r.y);
+            mod[e] = make_float2(-2.f * gam * r.x, 2.f * gam * r.y);
+            if (kx == 0) {
+                const float2 dn = I[(tc + 8 * e) * kDNH + kDN / 2];
+                const float2 rn = make_float2(dn.x - nyq[8 * e].x, dn.y - nyq[8 * e].y);
+                lacc += (double)(rn.x * rn.x + rn.y * rn.y);
+                nyq[8 * e] = make_float2(-2.f * gam * rn.x, 2.f * gam * rn.y);
             }
         }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) lacc += __shfl_xor_sync(0xffffffffu, lacc, off);
-        if (lane == 0) prm.unit_loss[u] = (double)gam * lacc;
-        __syncwarp();
-        if (!backward) continue;
+        if (lane == 0) part[w] = lacc;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0.0;
+            for (int q = 0; q < kDWarps; ++q) s += part[q];
+            prm.unit_loss[u] = (double)gam * s;
+        }
+        if (!backward) {
+            __syncthreads();  // part is free again
+            continue;
+        }
         // ------------------------------ g_i = F^H[conj(Phi_i) G] (real), per atom
-        float* const gobj = prm.unit_gobj;
-        if (gobj)
-            for (int e = lane; e < kDN * kDoLd; e += 32) DO[e] = 0.f;
-        for (int i = 0; i < prm.M; ++i) {
-            const float2* Phi = prm.atom_otf + (size_t)i * kDN * kDNH;
-            const float* ai = a + (size_t)i * kDN * kDN;
-            // the packed real columns: conj(V(ky, 0) + i V(ky, N/2)), two rows a lane
+        float s0[8], s1[8];  // the unit's share of dL/do
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int ky = lane + h * (kDN / 2);
-                const float2 va = cmul(cconj(Phi[ky * kDNH]), A[ky * kDES]);
-                const float2 vb = cmul(cconj(Phi[ky * kDNH + kDN / 2]), A[ky * kDES + kDN / 2]);
-                Z[ky] = make_float2(va.x - vb.y, -(va.y + vb.x));
-            }
-            __syncwarp();
-            // columns along ky: F^H x = conj(F conj x); lane 0 the packed columns
-            float2 v[kDN];
+        for (int e = 0; e < 8; ++e) s0[e] = s1[e] = 0.f;
+        for (int m = 0; m < prm.M; ++m) {
+            float2* E = buf0 + b * (kDN * kDS);
+            b ^= 1;
+            const float2* Phi = prm.atom_otf + (size_t)m * kDN * kDNH;
+            {
+                // columns along ky: F^H x = conj(F conj x); line 0 the packed real columns
+                const ColLine<kDN, kDS> ln{E + kx, shift};
+                float2 v[8], x[8];
 #pragma unroll
-            for (int ky = 0; ky < kDN; ++ky) {
-                const float2 vv = cmul(cconj(Phi[ky * kDNH + lane]), A[ky * kDES + lane]);
-                const float2 zz = Z[ky];
-                v[ky] = lane > 0 ? cconj(vv) : zz;
-            }
-            line_fft<kDN, -1>(v, 0);
+                for (int e = 0; e < 8; ++e) v[e] = cmul(Phi[(tc + 8 * e) * kDNH + kx], mod[e]);
+                if (kx == 0) {
 #pragma unroll
-            for (int ky = 0; ky < kDN; ++ky) E[ky * kDES + lane] = cconj(v[ky]);
-            __syncwarp();
-            // rows y and y + N/2: F^H of the Hermitian-extended rows, packed as
-            // T_y + i T_(y+N/2) (both results real)
-            const int y = lane;
-#pragma unroll
-            for (int x = 0; x < kDN; ++x) {
-                float2 p, q;
-                if (x == 0) {
-                    p = make_float2(E[y * kDES].x, 0.f);
-                    q = make_float2(E[(y + kDN / 2) * kDES].x, 0.f);
-                } else if (x == kDN / 2) {
-                    p = make_float2(E[y * kDES].y, 0.f);
-                    q = make_float2(E[(y + kDN / 2) * kDES].y, 0.f);
-                } else if (x < kDN / 2) {
-                    p = E[y * kDES + x];
-                    q = E[(y + kDN / 2) * kDES + x];
-                } else {
-                    p = cconj(E[y * kDES + kDN - x]);
-                    q = cconj(E[(y + kDN / 2) * kDES + kDN - x]);
+                    for (int e = 0; e < 8; ++e) {
+                        const float2 c = cmul(Phi[(tc + 8 * e) * kDNH + kDN / 2], nyq[8 * e]);
+                        v[e] = make_float2(v[e].x + c.y, v[e].y - c.x);
+                    }
                 }
-                v[x] = make_float2(p.x - q.y, -(p.y + q.x));  // conj(p + i q)
-            }
-            line_fft<kDN, -1>(v, 0);
-            // v[x].x = g_i(y, x), -v[x].y = g_i(y + N/2, x)
-            const float4* o0 = reinterpret_cast<const float4*>(o + y * kDN);
-            const float4* o1 = reinterpret_cast<const float4*>(o + (y + kDN / 2) * kDN);
-            const float4* a0 = reinterpret_cast<const float4*>(ai + y * kDN);
-            const float4* a1 = reinterpret_cast<const float4*>(ai + (y + kDN / 2) * kDN);
-            float4* gc0 = prm.grad_coeff ? reinterpret_cast<float4*>(prm.grad_coeff + ((size_t)u * prm.M + i) * kDN * kDN + y * kDN) : nullptr;
-            float4* gc1 = gc0 ? gc0 + (kDN / 2) * kDN / 4 : nullptr;
+                strided_to_blocked<kDN>(ln, v, x, LaneTwiddles<kDN>(table, tc), tc);
+                __syncwarp();
+                // rows y and y + N/2 of T = conj(x): conj of T_y + i T_(y+N/2) at kx, and its mirror
 #pragma unroll
-            for (int c = 0; c < kDN / 4; ++c) {
-                const float g0[4] = {v[4 * c].x, v[4 * c + 1].x, v[4 * c + 2].x, v[4 * c + 3].x};
-                const float g1[4] = {-v[4 * c].y, -v[4 * c + 1].y, -v[4 * c + 2].y, -v[4 * c + 3].y};
-                if (gc0) {
-                    const float4 p = o0[c], q = o1[c];
-                    gc0[c] = make_float4(p.x * g0[0], p.y * g0[1], p.z * g0[2], p.w * g0[3]);
-                    gc1[c] = make_float4(q.x * g1[0], q.y * g1[1], q.z * g1[2], q.w * g1[3]);
-                }
-                if (gobj) {
-                    const float4 s = a0[c], t = a1[c];
-                    float* d0 = DO + y * kDoLd + 4 * c;
-                    float* d1 = DO + (y + kDN / 2) * kDoLd + 4 * c;
-                    d0[0] = fmaf(s.x, g0[0], d0[0]);
-                    d0[1] = fmaf(s.y, g0[1], d0[1]);
-                    d0[2] = fmaf(s.z, g0[2], d0[2]);
-                    d0[3] = fmaf(s.w, g0[3], d0[3]);
-                    d1[0] = fmaf(t.x, g1[0], d1[0]);
-                    d1[1] = fmaf(t.y, g1[1], d1[1]);
-                    d1[2] = fmaf(t.z, g1[2], d1[2]);
-                    d1[3] = fmaf(t.w, g1[3], d1[3]);
+                for (int e = 0; e < 4; ++e) {
+                    const float2 u0 = x[e], u1 = x[e + 4];
+                    float2 lo = make_float2(u0.x + u1.y, u0.y - u1.x), hi = make_float2(u0.x - u1.y, -u0.y - u1.x);
+                    if (kx == 0) {
+                        lo = make_float2(u0.x, -u1.x);
+                        hi = make_float2(-u0.y, u1.y);
+                    }
+                    ln.block(e)[tc * kDS] = lo;
+                    ln.block(e + 4)[tc * kDS] = hi;
                 }
             }
-            __syncwarp();  // E and Z free for the next atom
+            __syncthreads();
+            const RowLine<kDN, kDS> ln{E + i * kDS};
+            float2 v[8], g[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = ln.block(e)[tr];
+            if (prm.unit_gobj) {
+                const float* am = a + (size_t)m * kDN * kDN;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    a0[e] = am[r0 + 8 * e];
+                    a1[e] = am[r1 + 8 * e];
+                }
+            }
+            strided_to_blocked<kDN>(ln, v, g, LaneTwiddles<kDN>(table, tr), tr);
+            // g.x = g_i(y, x), -g.y = g_i(y + N/2, x)
+            if (prm.grad_coeff) {
+                float* gc = prm.grad_coeff + ((size_t)u * prm.M + m) * kDN * kDN;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    gc[r0 + 8 * e] = o0[e] * g[e].x;
+                    gc[r1 + 8 * e] = -o1[e] * g[e].y;
+                }
+            }
+            if (prm.unit_gobj) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    s0[e] = fmaf(a0[e], g[e].x, s0[e]);
+                    s1[e] = fmaf(a1[e], -g[e].y, s1[e]);
+                }
+            }
         }
-        if (gobj) {
-            float* out = gobj + (size_t)u * kDN * kDN;
-            for (int e = lane; e < kDN * kDN; e += 32) out[e] = DO[(e / kDN) * kDoLd + (e % kDN)];
+        if (prm.unit_gobj) {
+            float* out = prm.unit_gobj + (size_t)u * kDN * kDN;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                out[r0 + 8 * e] = s0[e];
+                out[r1 + 8 * e] = s1[e];
+            }
         }
-        __syncwarp();
     }
 }
 
@@ -330,7 +337,7 @@ extern "C" int mfbd_dict_loss_grad(const mfbd_dict_desc* desc, const void* atom_
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(dict_unit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDictSmem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, dict_unit_kernel, 32, kDictSmem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, dict_unit_kernel, 32 * kDWarps, kDictSmem);
     if (e != cudaSuccess) return set_cuda_error(e, "mfbd_dict_loss_grad setup");
     if (per_sm < 1) return set_error(MFBD_ERR_UNSUPPORTED, "the dictionary kernel does not fit an SM");
     unsigned char* ws = static_cast<unsigned char*>(workspace);
@@ -349,7 +356,7 @@ extern "C" int mfbd_dict_loss_grad(const mfbd_dict_desc* desc, const void* atom_
     prm.unit_gobj = grad_object ? reinterpret_cast<float*>(ws + dict_gobj_offset(units)) : nullptr;
     long long ctas = (long long)sms * per_sm;
     if (ctas > units) ctas = units;
-    dict_unit_kernel<<<(int)ctas, 32, kDictSmem, s>>>(prm);
+    dict_unit_kernel<<<(int)ctas, 32 * kDWarps, kDictSmem, s>>>(prm);
     if ((e = cudaGetLastError()) != cudaSuccess) return set_cuda_error(e, "dict_unit_kernel launch");
     dict_combine_kernel<<<desc->n_patches, 256, 0, s>>>(prm.K, prm.J, prm.unit_loss, prm.unit_gobj, grad_object,
                                                         loss);
