@@ -55,6 +55,7 @@ struct mfbd_batch {
     BatchProblem* d_probs = nullptr;
     BatchItem* d_items = nullptr;
     int* d_ctr = nullptr;               // [patches][BC_COUNT], then 8 tickets, then the error flag
+    double* d_lpart = nullptr;          // [patches][kMaxRedParts]
     float* d_phi = nullptr;
     float* d_gphi = nullptr;
     float2* d_gscr = nullptr;
@@ -164,6 +165,31 @@ std::vector<BatchItem> build_items(const mfbd_batch* b, int mode, int window, st
     return items;
 }
 
+// The launch list: the items of build_items with P, R and G cut into their
+// parts (next to one another, so every dependency still precedes its
+// dependants).
+std::vector<BatchItem> launch_items(const mfbd_batch* b, int mode, int window, std::vector<int>* stage_begin) {
+    const std::vector<BatchItem> items = build_items(b, mode, window, stage_begin);
+    std::vector<BatchItem> out;
+    std::vector<int> start;  // of every item of build_items, then the end
+    for (const BatchItem& it : items) {
+        const BatchProblem& pr = b->probs[it.prob];
+        const int parts = it.kind == BK_PROJ   ? proj_parts(pr.K, pr.J)
+                          : it.kind == BK_RED  ? red_parts(pr.N)
+                          : it.kind == BK_GRAD ? grad_parts(pr.J, pr.M)
+                                               : 1;
+        start.push_back((int)out.size());
+        for (int q = 0; q < parts; ++q) {
+            out.push_back(it);
+            out.back().part = q;
+        }
+    }
+    start.push_back((int)out.size());
+    if (stage_begin)
+        for (int& s : *stage_begin) s = start[s];
+    return out;
+}
+
 int apply_schedule(mfbd_batch* b, int mode, int window, int ctas_per_sm, int variant) {
     if (mode != MFBD_BATCH_ONE_LAUNCH && mode != MFBD_BATCH_STAGED)
         return set_error(MFBD_ERR_INVALID_ARG, "unknown batch schedule mode");
@@ -173,7 +199,7 @@ int apply_schedule(mfbd_batch* b, int mode, int window, int ctas_per_sm, int var
     if (ctas_per_sm < 0 || ctas_per_sm > b->max_per_sm_v[variant])
         return set_error(MFBD_ERR_INVALID_ARG, "ctas_per_sm out of range for this batch");
     std::vector<int> sb;
-    std::vector<BatchItem> items = build_items(b, mode, window, &sb);
+    std::vector<BatchItem> items = launch_items(b, mode, window, &sb);
     if ((long long)items.size() != b->n_items) return set_error(MFBD_ERR_STATE, "item count changed");
     if (!items.empty()) {
         cudaError_t e =
@@ -210,6 +236,7 @@ int run_batch(mfbd_batch_t b, const float* coeffs, const void* spectra, double* 
     prm.kinds = kinds;
     prm.half_box = b->half_box;
     prm.ctr = b->d_ctr;
+    prm.lpart = b->d_lpart;
     prm.err = b->d_ctr + ctr_ints;
     prm.coeffs = coeffs;
     prm.spectra = static_cast<const float2*>(spectra);
@@ -470,10 +497,11 @@ int mfbd_batch_create(mfbd_batch_t* out, const mfbd_plan_desc* problems, int n_p
         if ((st = balloc(b, &b->d_gphi, (size_t)phi))) throw st;
         if ((st = balloc(b, &b->d_gscr, (size_t)gscr))) throw st;
         if ((st = balloc(b, &b->d_pscr, (size_t)pscr))) throw st;
+        if ((st = balloc(b, &b->d_lpart, (size_t)b->patches * kMaxRedParts))) throw st;
         if ((st = balloc(b, &b->d_ctr, (size_t)b->patches * BC_COUNT + 9))) throw st;
         if ((e = cudaMemsetAsync(b->d_ctr, 0, ((size_t)b->patches * BC_COUNT + 9) * sizeof(int), s)))
             throw set_cuda_error(e, "clear batch counters");
-        b->n_items = (long long)build_items(b, MFBD_BATCH_ONE_LAUNCH, 0, nullptr).size();
+        b->n_items = (long long)launch_items(b, MFBD_BATCH_ONE_LAUNCH, 0, nullptr).size();
         if (b->n_items > (1ll << 30)) throw set_error(MFBD_ERR_UNSUPPORTED, "too many work items in one batch");
         if ((st = balloc(b, &b->d_items, (size_t)std::max(1ll, b->n_items)))) throw st;
         if ((e = cudaStreamSynchronize(s))) throw set_cuda_error(e, "batch upload");

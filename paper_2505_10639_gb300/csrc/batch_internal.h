@@ -63,11 +63,13 @@ struct BatchItem {
     int patch;      // patch within the problem
     int kj;         // F, A: k * J + j of the first unit; P, R, G: 0
     int extra;      // F, A: further units kj + 1 .. kj + extra in the item (N <= 64: 0 .. kSmallUnits - 1)
-    int pad[3];
+    int part;       // P, R, G: which of the item's parts (each a work item of the launch list)
+    int pad[2];
 };
 
-// Dependency counters of a patch (cleared before every launch).
-enum BatchCtr : int { BC_PROJ = 0, BC_FWD = 1, BC_RED = 2, BC_ADJ = 3, BC_COUNT = 4 };
+// Dependency counters of a patch (cleared before every launch); BC_LOSS: R
+// parts whose share of the loss is written.
+enum BatchCtr : int { BC_PROJ = 0, BC_FWD = 1, BC_RED = 2, BC_ADJ = 3, BC_LOSS = 4, BC_COUNT = 5 };
 
 struct BatchParams {
     const BatchProblem* probs;
@@ -78,6 +80,7 @@ struct BatchParams {
     int kinds;              // bit k set: items of kind k run (the others are skipped, and signalled)
     bool half_box;          // every pupil box at most N/2 px
     int* ctr;               // [patches][BC_COUNT] counters
+    double* lpart;          // [patches][kMaxRedParts] losses of the R parts
     int* ticket;            // next item to take
     int* err;               // set when a dependency wait gives up
     const float* coeffs;
@@ -93,8 +96,21 @@ struct BatchParams {
 
 constexpr int kBT = 256;        // threads per CTA of the batch kernel
 constexpr int kJC = 8;          // frames per register tile of its P and G items
+constexpr int kGM = 32;         // modes per G part
+constexpr int kMaxRedParts = 4;
 constexpr int kSmallUnits = 2;  // units of an F or A item of N <= 64
 constexpr int kBatchTwiddles = 96 + 64 + 192 + 128;  // complex elements of the four tables
+
+// Parts of a patch's items. The P, R and G items of a patch are cut so that a
+// few hundred large patches fill the SMs: P by object and tile of kJC frames,
+// R by about 2,048 frequencies of each object, G by tiles of kJC frames and
+// kGM modes.
+__host__ __device__ inline int proj_parts(int K, int J) { return K * ((J + kJC - 1) / kJC); }
+__host__ __device__ inline int red_parts(int N) {
+    const int n = N * (N / 2 + 1) / 2048;
+    return n < 1 ? 1 : n > kMaxRedParts ? kMaxRedParts : n;
+}
+__host__ __device__ inline int grad_parts(int J, int M) { return ((J + kJC - 1) / kJC) * ((M + kGM - 1) / kGM); }
 
 // Dynamic shared memory for a batch holding the patch sizes (48, 64, 96, 128)
 // that are set in `sizes`.

@@ -7,8 +7,9 @@
 namespace mfbd_dev {
 
 size_t batch_smem(const bool (&sizes)[4], bool half_box) {
-    // the twiddles, then the exchange buffers of an item or the P item's coefficient tile
-    size_t unit = kJC * 256 * sizeof(float) / sizeof(float2);
+    // the twiddles, then the exchange buffers of an item, a P part's coefficient
+    // tile (up to 256 modes) or a G part's sums
+    size_t unit = (size_t)kJC * std::max(256, kBT / 32 * kGM) * sizeof(float) / sizeof(float2);
     const int n[4] = {48, 64, 96, 128};
     for (int i = 0; i < 4; ++i)
         if (sizes[i])

@@ -2,7 +2,8 @@
 // problems (patch sizes 48, 64, 96, 128; objects, frames and modes per
 // problem) in one launch.
 //
-// The work is a list of items, each of one kind (BatchKind): P, the phases
+// The work is a list of items, each of one kind (BatchKind), those of a whole
+// patch cut into parts: P, the phases
 // phi = c_k B_k a of every object and frame of a patch (Sec. 3.1, Eq. 22);
 // F, the forward passes of a unit (Eqs. 20-21 and the OTF); R, the frame
 // reduction of a patch (Sec. 2.2.1, Eqs. 11-12, and the adjoint seeds); A,
@@ -129,109 +130,115 @@ __device__ void item_unit(const BatchParams& prm, const BatchProblem& pr, const 
     else run(CtaBar{});
 }
 
-// P item: phi_kj[i] = c_k sum_m a_j[m] B_k[m][i] on every box pixel i, for
-// every object and frame of the patch; kJC frames per register tile with
-// their coefficients staged in shared memory mode-major ([m][kJC]: two
-// 16-byte loads per mode).
-__device__ void item_proj(const BatchParams& prm, const BatchProblem& pr, int p, float* sa) {
+// P part: phi_kj[i] = c_k sum_m a_j[m] B_k[m][i] on every box pixel i for one
+// object and kJC frames of the patch, their coefficients staged in shared
+// memory mode-major ([m][kJC]: two 16-byte loads per mode).
+__device__ void item_proj(const BatchParams& prm, const BatchProblem& pr, int p, int part, float* sa) {
     const int t = threadIdx.x, J = pr.J, M = pr.M;
+    const int k = part % pr.K, jc = part / pr.K * kJC, nj = min(kJC, J - jc);
     const float* a = prm.coeffs + pr.coeff_off + (size_t)p * J * M;
-    for (int jc = 0; jc < J; jc += kJC) {
-        const int nj = min(kJC, J - jc);
-        __syncthreads();
-        for (int e = t; e < kJC * M; e += kBT) {
-            const int m = e / kJC, jj = e - m * kJC;
-            sa[e] = jj < nj ? a[(size_t)(jc + jj) * M + m] : 0.f;
-        }
-        __syncthreads();
-        const float4* sa4 = reinterpret_cast<const float4*>(sa);
-        for (int k = 0; k < pr.K; ++k) {
-            const BatchObj& ob = pr.obj[k];
-            const int npix = ob.W * ob.W;
-            const long long us = unit_stride_phi(ob.W);
-            float* phi = prm.phi + pr.phi_off + (long long)p * pr.phi_patch + ob.phi_koff + jc * us;
-            for (int i = t; i < npix; i += kBT) {
-                float acc[kJC];
-#pragma unroll
-                for (int jj = 0; jj < kJC; ++jj) acc[jj] = 0.f;
-                for (int m = 0; m < M; ++m) {
-                    const float b = ob.bm[(size_t)m * npix + i];
-                    const float4 c0 = sa4[2 * m], c1 = sa4[2 * m + 1];
-                    acc[0] = fmaf(c0.x, b, acc[0]);
-                    acc[1] = fmaf(c0.y, b, acc[1]);
-                    acc[2] = fmaf(c0.z, b, acc[2]);
-                    acc[3] = fmaf(c0.w, b, acc[3]);
-                    acc[4] = fmaf(c1.x, b, acc[4]);
-                    acc[5] = fmaf(c1.y, b, acc[5]);
-                    acc[6] = fmaf(c1.z, b, acc[6]);
-                    acc[7] = fmaf(c1.w, b, acc[7]);
-                }
-#pragma unroll
-                for (int jj = 0; jj < kJC; ++jj)
-                    if (jj < nj) phi[jj * us + i] = ob.scale * acc[jj];
-            }
-        }
+    for (int e = t; e < kJC * M; e += kBT) {
+        const int m = e / kJC, jj = e - m * kJC;
+        sa[e] = jj < nj ? a[(size_t)(jc + jj) * M + m] : 0.f;
     }
-}
-
-// G item: grad[j][m] = sum_k c_k sum_i dL/dphi_kj[i] B_k[m][i], the objects
-// added in order; one thread per (mode, tile of kJC frames). (Staging
-// dL/dphi and basis chunks in shared memory was measured slower: 5.7 against
-// 2.0 ms for the 2000-problem batch.)
-__device__ void item_grad(const BatchParams& prm, const BatchProblem& pr, int p) {
-    const int t = threadIdx.x, J = pr.J, M = pr.M;
-    const int tiles = (J + kJC - 1) / kJC;
-    float* grad = prm.grad + pr.coeff_off + (size_t)p * J * M;
-    for (int idx = t; idx < M * tiles; idx += kBT) {
-        const int m = idx % M, jc = (idx / M) * kJC, nj = min(kJC, J - jc);
+    __syncthreads();
+    const float4* sa4 = reinterpret_cast<const float4*>(sa);
+    const BatchObj& ob = pr.obj[k];
+    const int npix = ob.W * ob.W;
+    const long long us = unit_stride_phi(ob.W);
+    float* phi = prm.phi + pr.phi_off + (long long)p * pr.phi_patch + ob.phi_koff + jc * us;
+    for (int i = t; i < npix; i += kBT) {
         float acc[kJC];
 #pragma unroll
         for (int jj = 0; jj < kJC; ++jj) acc[jj] = 0.f;
-        for (int k = 0; k < pr.K; ++k) {
-            const BatchObj& ob = pr.obj[k];
-            const int npix = ob.W * ob.W;
-            const long long us = unit_stride_phi(ob.W);
-            const float* g = prm.gphi + pr.phi_off + (long long)p * pr.phi_patch + ob.phi_koff + jc * us;
-            const float* row[kJC];
-#pragma unroll
-            for (int jj = 0; jj < kJC; ++jj) row[jj] = g + min(jj, nj - 1) * us;
-            float part[kJC];
-#pragma unroll
-            for (int jj = 0; jj < kJC; ++jj) part[jj] = 0.f;
-            // four pixels per step: one 16-byte load of each frame's dL/dphi
-            // (rows are 256-byte aligned), then the tail
-            const int n4 = npix & ~3;
-            for (int i = 0; i < n4; i += 4) {
-                const float b0 = ob.bt[(size_t)i * ob.ldt + m], b1 = ob.bt[(size_t)(i + 1) * ob.ldt + m];
-                const float b2 = ob.bt[(size_t)(i + 2) * ob.ldt + m], b3 = ob.bt[(size_t)(i + 3) * ob.ldt + m];
-#pragma unroll
-                for (int jj = 0; jj < kJC; ++jj) {
-                    const float4 gv = *reinterpret_cast<const float4*>(row[jj] + i);
-                    float x = fmaf(gv.x, b0, part[jj]);
-                    x = fmaf(gv.y, b1, x);
-                    x = fmaf(gv.z, b2, x);
-                    part[jj] = fmaf(gv.w, b3, x);
-                }
-            }
-            for (int i = n4; i < npix; ++i) {
-                const float b = ob.bt[(size_t)i * ob.ldt + m];
-#pragma unroll
-                for (int jj = 0; jj < kJC; ++jj) part[jj] = fmaf(row[jj][i], b, part[jj]);
-            }
-#pragma unroll
-            for (int jj = 0; jj < kJC; ++jj) acc[jj] = fmaf(ob.scale, part[jj], acc[jj]);
+#pragma unroll 8
+        for (int m = 0; m < M; ++m) {
+            const float b = ob.bm[(size_t)m * npix + i];
+            const float4 c0 = sa4[2 * m], c1 = sa4[2 * m + 1];
+            acc[0] = fmaf(c0.x, b, acc[0]);
+            acc[1] = fmaf(c0.y, b, acc[1]);
+            acc[2] = fmaf(c0.z, b, acc[2]);
+            acc[3] = fmaf(c0.w, b, acc[3]);
+            acc[4] = fmaf(c1.x, b, acc[4]);
+            acc[5] = fmaf(c1.y, b, acc[5]);
+            acc[6] = fmaf(c1.z, b, acc[6]);
+            acc[7] = fmaf(c1.w, b, acc[7]);
         }
 #pragma unroll
         for (int jj = 0; jj < kJC; ++jj)
-            if (jj < nj) grad[(size_t)(jc + jj) * M + m] = acc[jj];
+            if (jj < nj) phi[jj * us + i] = ob.scale * acc[jj];
     }
 }
 
-// R item: the CTA's threads share each object's frequencies; the patch loss
-// adds an object's warps in order, then the objects in order.
+// G part: grad[j][m] = sum_k c_k sum_i dL/dphi_kj[i] B_k[m][i] for kJC frames
+// and kGM modes (one per lane), the objects added in order. The warps take an
+// eighth of an object's pixels each and add their sums in warp order through
+// shared memory (kBT / 32 x kJC x kGM floats).
+__device__ void item_grad(const BatchParams& prm, const BatchProblem& pr, int p, int part, float* sums) {
+    constexpr int kW = kBT / 32;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, J = pr.J, M = pr.M;
+    const int mt = (M + kGM - 1) / kGM, jc = part / mt * kJC, nj = min(kJC, J - jc);
+    const int m0 = part % mt * kGM, m = min(m0 + lane, M - 1);
+    float acc[kJC];
+#pragma unroll
+    for (int jj = 0; jj < kJC; ++jj) acc[jj] = 0.f;
+    for (int k = 0; k < pr.K; ++k) {
+        const BatchObj& ob = pr.obj[k];
+        const int npix = ob.W * ob.W;
+        const long long us = unit_stride_phi(ob.W);
+        const float* g = prm.gphi + pr.phi_off + (long long)p * pr.phi_patch + ob.phi_koff + jc * us;
+        const float* row[kJC];
+#pragma unroll
+        for (int jj = 0; jj < kJC; ++jj) row[jj] = g + min(jj, nj - 1) * us;
+        const float* bt = ob.bt + m;
+        float sum[kJC];
+#pragma unroll
+        for (int jj = 0; jj < kJC; ++jj) sum[jj] = 0.f;
+        // four pixels per step: one 16-byte load of each frame's dL/dphi (rows
+        // are 256-byte aligned), the same for all lanes; then the tail
+        const int n4 = npix & ~3, per = (n4 / 4 + kW - 1) / kW * 4;
+        const int i1 = min(n4, (w + 1) * per);
+#pragma unroll 2
+        for (int i = w * per; i < i1; i += 4) {
+            const float b0 = bt[(size_t)i * ob.ldt], b1 = bt[(size_t)(i + 1) * ob.ldt];
+            const float b2 = bt[(size_t)(i + 2) * ob.ldt], b3 = bt[(size_t)(i + 3) * ob.ldt];
+#pragma unroll
+            for (int jj = 0; jj < kJC; ++jj) {
+                const float4 gv = *reinterpret_cast<const float4*>(row[jj] + i);
+                float x = fmaf(gv.x, b0, sum[jj]);
+                x = fmaf(gv.y, b1, x);
+                x = fmaf(gv.z, b2, x);
+                sum[jj] = fmaf(gv.w, b3, x);
+            }
+        }
+        if (w == kW - 1)
+            for (int i = n4; i < npix; ++i) {
+                const float b = bt[(size_t)i * ob.ldt];
+#pragma unroll
+                for (int jj = 0; jj < kJC; ++jj) sum[jj] = fmaf(row[jj][i], b, sum[jj]);
+            }
+#pragma unroll
+        for (int jj = 0; jj < kJC; ++jj) acc[jj] = fmaf(ob.scale, sum[jj], acc[jj]);
+    }
+#pragma unroll
+    for (int jj = 0; jj < kJC; ++jj) sums[(w * kJC + jj) * kGM + lane] = acc[jj];
+    __syncthreads();
+    float* grad = prm.grad + pr.coeff_off + (size_t)p * J * M;
+    for (int e = threadIdx.x; e < kJC * kGM; e += kBT) {
+        const int jj = e / kGM, mm = m0 + e % kGM;
+        float v = 0.f;
+#pragma unroll
+        for (int q = 0; q < kW; ++q) v += sums[q * kJC * kGM + e];
+        if (jj < nj && mm < M) grad[(size_t)(jc + jj) * M + mm] = v;
+    }
+}
+
+// R part: the CTA's threads share the part's frequencies of each object; the
+// patch loss adds an object's warps in order, then the objects, then (the last
+// part to arrive) the parts.
 template <int HOLD>
-__device__ void item_reduce(const BatchParams& prm, const BatchProblem& pr, int p, double* part) {
-    const int N = pr.N, NH = N / 2 + 1, J = pr.J;
+__device__ void item_reduce(const BatchParams& prm, const BatchProblem& pr, int p, int part, double* warps) {
+    const int N = pr.N, NH = N / 2 + 1, J = pr.J, parts = red_parts(N);
     const size_t dstride = (size_t)N * NH;
     double tot = 0.0;
     for (int k = 0; k < pr.K; ++k) {
@@ -247,10 +254,22 @@ __device__ void item_reduce(const BatchParams& prm, const BatchProblem& pr, int 
         r.supp = pr.obj[k].supp;
         r.sw = pr.sw;
         r.obj = prm.object ? prm.object + pr.obj_off + ((size_t)p * pr.K + k) * dstride : nullptr;
-        tot += cta_sum<kBT / 32>(reduce_lane<HOLD>(r, threadIdx.x, kBT), part);
+        tot += cta_sum<kBT / 32>(reduce_lane<HOLD>(r, kBT * part + threadIdx.x, kBT * parts), warps);
         __syncthreads();
     }
-    if (threadIdx.x == 0) prm.loss[pr.loss_off + p] = tot;
+    if (threadIdx.x == 0) {
+        if (parts > 1) {
+            const long long patch = pr.ctr_off + p;
+            volatile double* lp = prm.lpart + patch * kMaxRedParts;
+            lp[part] = tot;
+            __threadfence();
+            if (atomicAdd(prm.ctr + patch * BC_COUNT + BC_LOSS, 1) != parts - 1) return;
+            __threadfence();
+            tot = 0.0;
+            for (int i = 0; i < parts; ++i) tot += lp[i];
+        }
+        prm.loss[pr.loss_off + p] = tot;
+    }
 }
 
 template <bool HALF, bool ADJ>
@@ -276,7 +295,8 @@ __global__ void __launch_bounds__(kBT, MINB) batch_kernel(const BatchParams prm)
     load_twiddles<96>(smem + kTwOff<96>, threadIdx.x, kBT);
     load_twiddles<128>(smem + kTwOff<128>, threadIdx.x, kBT);
     __shared__ int s_item, s_ok;
-    __shared__ double part[kBT / 32];
+    __shared__ double warps[kBT / 32];
+    float* scratch = reinterpret_cast<float*>(smem + kBatchTwiddles);  // of the P and G parts
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(prm.ticket, 1);
         __syncthreads();
@@ -290,9 +310,9 @@ __global__ void __launch_bounds__(kBT, MINB) batch_kernel(const BatchParams prm)
             if (prm.wait) {
                 const int units = pr.K * pr.J;
                 switch (it.kind) {
-                    case BK_FWD: ok = wait_ctr(ctr + BC_PROJ, 1, prm.err); break;
+                    case BK_FWD: ok = wait_ctr(ctr + BC_PROJ, proj_parts(pr.K, pr.J), prm.err); break;
                     case BK_RED: ok = wait_ctr(ctr + BC_FWD, units, prm.err); break;
-                    case BK_ADJ: ok = wait_ctr(ctr + BC_RED, 1, prm.err); break;
+                    case BK_ADJ: ok = wait_ctr(ctr + BC_RED, red_parts(pr.N), prm.err); break;
                     case BK_GRAD: ok = wait_ctr(ctr + BC_ADJ, units, prm.err); break;
                     default: break;
                 }
@@ -302,11 +322,11 @@ __global__ void __launch_bounds__(kBT, MINB) batch_kernel(const BatchParams prm)
         __syncthreads();
         if (s_ok && ((prm.kinds >> it.kind) & 1)) {
             switch (it.kind) {
-                case BK_PROJ: item_proj(prm, pr, it.patch, reinterpret_cast<float*>(smem + kBatchTwiddles)); break;
+                case BK_PROJ: item_proj(prm, pr, it.patch, it.part, scratch); break;
                 case BK_FWD: dispatch_unit<HALF, false>(prm, pr, it, smem); break;
-                case BK_RED: item_reduce<MINB == 2 ? 16 : 8>(prm, pr, it.patch, part); break;
+                case BK_RED: item_reduce<MINB == 2 ? 16 : 8>(prm, pr, it.patch, it.part, warps); break;
                 case BK_ADJ: dispatch_unit<HALF, true>(prm, pr, it, smem); break;
-                default: item_grad(prm, pr, it.patch); break;
+                default: item_grad(prm, pr, it.patch, it.part, scratch); break;
             }
         }
         __syncthreads();  // the item's writes precede the signal; s_item is free again
