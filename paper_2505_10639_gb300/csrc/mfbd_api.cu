@@ -257,6 +257,27 @@ void release(mfbd_plan* p) {
     p->allocations.clear();
 }
 
+// 64 px: whether mfbd_loss_grad runs the fused kernel (its frames and pupil
+// boxes fit) or the caller asked for the pass machine's three kernels. The
+// other 64 px plans (more than 12 frames, boxes over 37 px) run the general
+// sizes' kernels: 6,750 units of 15 frames, forward + reduction + adjoint 0.148
+// + 0.068 + 0.133 ms on the pass machine, 0.100 + 0.075 + 0.138 on those.
+bool fused_or_split(const mfbd_plan_desc* d) {
+    if (d->flags & MFBD_FLAG_SPLIT_PASSES) return true;
+    int box = 1;
+    for (int k = 0; k < d->n_objects; ++k) {
+        const std::vector<uint8_t> mask = mfbd_host::pupil_mask(d->n_pix, d->pupil_diam_px[k], d->central_obscuration);
+        int lo = d->n_pix, hi = -1;
+        for (int i = 0; i < d->n_pix * d->n_pix; ++i)
+            if (mask[i]) {
+                lo = std::min(lo, std::min(i % d->n_pix, i / d->n_pix));
+                hi = std::max(hi, std::max(i % d->n_pix, i / d->n_pix));
+            }
+        box = std::max(box, hi - lo + 1);
+    }
+    return fused_pair_supported(d->n_frames, fused_geometry(box).xs);
+}
+
 // Kernel parameters for patches [p0, p0 + np): spectra, loss and object
 // point at patch p0; the per-unit scratch is reused from its start.
 FusedParams fused_params(const mfbd_plan* p, int p0, int np, const void* spectra, double* loss, void* object,
@@ -692,7 +713,8 @@ int mfbd_plan_create(mfbd_plan_t* out, const mfbd_plan_desc* d, void* stream) {
     p->M = d->n_modes;
     p->flags = d->flags;
     p->precision = d->precision;
-    p->generic = d->n_pix != kN || (d->flags & (MFBD_FLAG_RECOMPUTE_BACKWARD | MFBD_FLAG_GENERIC_KERNELS));
+    p->generic = d->n_pix != kN || (d->flags & (MFBD_FLAG_RECOMPUTE_BACKWARD | MFBD_FLAG_GENERIC_KERNELS)) ||
+                 !fused_or_split(d);
     p->gamma = d->gamma;
     p->device = dev;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
