@@ -254,7 +254,16 @@ __device__ void item_reduce(const BatchParams& prm, const BatchProblem& pr, int 
         r.supp = pr.obj[k].supp;
         r.sw = pr.sw;
         r.obj = prm.object ? prm.object + pr.obj_off + ((size_t)p * pr.K + k) * dstride : nullptr;
-        tot += cta_sum<kBT / 32>(reduce_lane<HOLD>(r, kBT * part + threadIdx.x, kBT * parts), warps);
+        auto share = [&](auto fs, auto hold) {
+            constexpr int FS = decltype(fs)::value, kF = 32 / FS;
+            return reduce_lane<decltype(hold)::value, FS>(r, kF * (kBT / 32 * part + (threadIdx.x >> 5)),
+                                                          kF * (kBT / 32) * parts);
+        };
+        using fftreg::IC;
+        const double v = J <= HOLD       ? share(IC<1>{}, IC<HOLD>{})
+                         : J <= 2 * HOLD ? share(IC<2>{}, IC<HOLD>{})
+                                         : share(IC<1>{}, IC<0>{});
+        tot += cta_sum<kBT / 32>(v, warps);
         __syncthreads();
     }
     if (threadIdx.x == 0) {

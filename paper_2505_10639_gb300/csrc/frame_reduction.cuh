@@ -38,35 +38,45 @@ struct RedPtr {
     float2* gobj = nullptr;          // with oin: dL/dconj(O) [N][spec_ld], or null
 };
 
-// Lanes take the frequencies f0, f0 + fstep, ...; the returned sum covers
-// this lane's. Outside the OTF support H vanishes and G with it: neither is
-// read or written there (the passes of the larger sizes do not store or load
-// them either), which at pupils of 0.35 to 0.5 N px leaves 40 to 80 % of the
-// half spectrum.
+// One warp takes the 32 / FS frequencies f0, f0 + 1, ... and then every fstep
+// further on; lane q (32 / FS) + i holds frames q ceil(J / FS), ... of
+// frequency i, and the FS lanes of a frequency add their sums by shuffles. The
+// returned sum covers the lane's share. Outside the OTF support H vanishes and
+// G with it: neither is read or written there (the passes of the larger sizes
+// do not store or load them either), which at pupils of 0.35 to 0.5 N px leaves
+// 40 to 80 % of the half spectrum.
 //
 // HBM is the floor (D once, H and G once on the support); what it needs is
-// loads in flight. For J <= HOLD a frequency's frames are loaded once, all at
-// once, into registers; otherwise in chunks of kChunk frames, twice (the second
-// time from L2). Lanes outside the support take the same way with their loads
-// of H predicated off: a path of their own, which most warps would run as well
-// as the other, was slower (96 px 0.081 -> 0.100 ms).
-template <int HOLD>
+// loads in flight and no second read: a frequency's frames are loaded once, all
+// at once, into the registers of its lanes (J <= HOLD FS), or (HOLD = 0, any J)
+// in chunks of kChunk frames, twice. Lanes outside the support take the same
+// way with their loads of H predicated off: a path of their own, which most
+// warps would run as well as the other, was slower (96 px 0.081 -> 0.100 ms).
+// The object-inferring loss (r.oin) needs FS = 1.
+template <int HOLD, int FS>
 __device__ __forceinline__ double reduce_lane(const RedPtr& r, int f0, int fstep) {
-    constexpr int kChunk = 8;
+    static_assert(FS == 1 || HOLD > 0, "frames are split over lanes in the register form only");
+    constexpr int kChunk = 8, kF = 32 / FS;
     const int N = r.N, NH = N / 2 + 1, half = N * NH, J = r.J;
     const unsigned dstride = (unsigned)N * r.spec_ld;  // J * dstride < 2^32
     const float gam = (float)r.gamma;
+    const int lane = threadIdx.x & 31, q = FS > 1 ? lane / kF : 0;
+    const int jq = (J + FS - 1) / FS, jb = q * jq, nj = FS > 1 ? max(0, min(jq, J - jb)) : J;  // this lane's frames
     KahanSum acc;
-    for (int f = f0; f < half; f += fstep) {
+    for (int fb = f0; fb < half; fb += fstep) {
+        const bool live = fb + lane % kF < half;
+        if (FS == 1 && !live) break;
+        const int f = live ? fb + lane % kF : half - 1;
         const int ky = f / NH, kx = f - ky * NH;
         const size_t doff = (size_t)ky * r.spec_ld + kx;
-        const float2* dp = r.d + doff;
-        float2* hp = r.h + f;
+        const float2 *dp0 = r.d + doff, *dp = dp0 + (unsigned)jb * dstride;
+        float2 *hp0 = r.h + f, *hp = hp0 + (unsigned)jb * (unsigned)half;
+        const float* wp = r.w + jb;
         const bool sup = wbit(r.supp, r.sw, ky, kx), seed = sup && f != 0;
         const float twice = (kx == 0 || kx == N / 2) ? 1.f : 2.f;
-        float2 o = r.oin ? r.oin[doff] : make_float2(0.f, 0.f), g = make_float2(gam * o.x, gam * o.y);
+        float2 o = FS == 1 && r.oin ? r.oin[doff] : make_float2(0.f, 0.f), g = make_float2(gam * o.x, gam * o.y);
         float t = 0.f;
-        if (r.oin && sup) {  // object-inferring loss: the object is given
+        if (FS == 1 && r.oin && sup) {  // object-inferring loss: the object is given
             t = explicit_frequency(J, dp, dstride, hp, half, r.w, r.gamma, seed, o, g);
         } else {
             float2 num = make_float2(0.f, 0.f);
@@ -80,11 +90,19 @@ __device__ __forceinline__ double reduce_lane(const RedPtr& r, int f0, int fstep
             auto scatter = [&](float2 d, float2 h, float wj, int j) {
                 const float2 res = csub(d, cmul(o, h));
                 t += wj * (res.x * res.x + res.y * res.y);
-                if (sup) hp[(unsigned)j * (unsigned)half] = seed ? cscale(cmul(cconj(o), res), -wj) : make_float2(0.f, 0.f);
+                if (sup && live)
+                    hp[(unsigned)j * (unsigned)half] = seed ? cscale(cmul(cconj(o), res), -wj) : make_float2(0.f, 0.f);
             };
             // false where the residual cancels (seed frequencies only)
             auto solve = [&]() {
-                if (r.oin) return true;  // outside the support: the data's energy, O as given
+                if (FS == 1 && r.oin) return true;  // outside the support: the data's energy, O as given
+#pragma unroll
+                for (int off = kF; off < 32; off <<= 1) {
+                    num.x += __shfl_xor_sync(0xffffffffu, num.x, off);
+                    num.y += __shfl_xor_sync(0xffffffffu, num.y, off);
+                    e += __shfl_xor_sync(0xffffffffu, e, off);
+                    qs += __shfl_xor_sync(0xffffffffu, qs, off);
+                }
                 qs += gam;
                 const float invq = 1.0f / qs;
                 o = cscale(num, invq);
@@ -92,25 +110,24 @@ __device__ __forceinline__ double reduce_lane(const RedPtr& r, int f0, int fstep
                 return !(seed && t_est < kCancel * e);
             };
             bool fine;
-            if (HOLD > 0 && J <= HOLD) {
-                constexpr int H = HOLD > 0 ? HOLD : 1;
-                float2 d[H], h[H];
-                float wv[H];
+            if constexpr (HOLD > 0) {
+                float2 d[HOLD], h[HOLD];
+                float wv[HOLD];
 #pragma unroll
-                for (int j = 0; j < H; ++j) {
-                    const bool in = j < J;
+                for (int j = 0; j < HOLD; ++j) {
+                    const bool in = j < nj;
                     d[j] = in ? dp[(unsigned)j * dstride] : make_float2(0.f, 0.f);
                     h[j] = in && sup ? hp[(unsigned)j * (unsigned)half] : make_float2(0.f, 0.f);
-                    wv[j] = in ? r.w[j] : 0.f;
+                    wv[j] = in ? wp[j] : 0.f;
                 }
 #pragma unroll
-                for (int j = 0; j < H; ++j)
-                    if (j < J) gather(d[j], h[j], wv[j]);
+                for (int j = 0; j < HOLD; ++j)
+                    if (j < nj) gather(d[j], h[j], wv[j]);
                 fine = solve();
                 if (fine) {
 #pragma unroll
-                    for (int j = 0; j < H; ++j)
-                        if (j < J) scatter(d[j], h[j], wv[j], j);
+                    for (int j = 0; j < HOLD; ++j)
+                        if (j < nj) scatter(d[j], h[j], wv[j], j);
                 }
             } else {
                 auto chunks = [&](bool on, auto&& use) {
@@ -123,7 +140,7 @@ __device__ __forceinline__ double reduce_lane(const RedPtr& r, int f0, int fstep
                             const bool in = on && j0 + c < J;
                             d[c] = in ? dp[(unsigned)(j0 + c) * dstride] : make_float2(0.f, 0.f);
                             h[c] = in && sup ? hp[(unsigned)(j0 + c) * (unsigned)half] : make_float2(0.f, 0.f);
-                            wv[c] = in ? r.w[j0 + c] : 0.f;
+                            wv[c] = in ? wp[j0 + c] : 0.f;
                         }
 #pragma unroll
                         for (int c = 0; c < kChunk; ++c)
@@ -137,15 +154,21 @@ __device__ __forceinline__ double reduce_lane(const RedPtr& r, int f0, int fstep
                     if (!sup) t = e;
                 }
             }
-            if (!fine) fp64_frequency(J, dp, dstride, hp, half, r.w, r.gamma, true, t, o);
-            else t += gam * (o.x * o.x + o.y * o.y);
+            if (!fine) {
+                t = 0.f;
+                if (q == 0 && live) fp64_frequency(J, dp0, dstride, hp0, half, r.w, r.gamma, true, t, o);
+            } else if (q == 0) {
+                t += gam * (o.x * o.x + o.y * o.y);
+            }
         }
+        if (!live) continue;
         acc.add(twice * t);
+        if (q != 0) continue;
         if (r.obj) {
             r.obj[doff] = o;
             if (r.spec_ld == N && kx > 0 && kx < N / 2) r.obj[(size_t)((N - ky) % N) * N + (N - kx)] = cconj(o);
         }
-        if (r.gobj) {
+        if (FS == 1 && r.gobj) {
             r.gobj[doff] = g;
             if (r.spec_ld == N && kx > 0 && kx < N / 2) r.gobj[(size_t)((N - ky) % N) * N + (N - kx)] = cconj(g);
         }

@@ -15,14 +15,15 @@ using namespace reduction;
 // A CTA takes 1/S of the frequencies of one (patch, object) at a time (S =
 // rsplit); with one object and one split its sum is the patch's loss,
 // otherwise the sums of a patch's objects and splits are added in order by
-// loss_combine_kernel. HOLD: frames of a frequency held in registers. Against
+// loss_combine_kernel. HOLD frames of a frequency are held by each of FS lanes. Against
 // one warp per (patch, object, split) and four frames' loads in flight: 2,904
 // units of 96 px 0.126 -> 0.081 ms, 735 of 128 px 0.085 -> 0.056, 12,800 of 128
-// px 0.852 -> 0.460 (58 % of the copy peak on what it cannot do without).
+// px 0.852 -> 0.442 (60 % of the copy peak on what it cannot do without).
 constexpr int kRedWarps = 8;
 
-template <int HOLD>
+template <int HOLD, int FS>
 __global__ void __launch_bounds__(32 * kRedWarps, HOLD == 32 ? 1 : 2) generic_reduce_kernel(const GenericParams prm) {
+    constexpr int kF = 32 / FS;  // frequencies of a warp
     __shared__ double part[kRedWarps];
     const int N = prm.N, half = N * (N / 2 + 1), J = prm.J, S = prm.rsplit;
     const size_t dstride = (size_t)N * prm.spec_ld;
@@ -44,7 +45,7 @@ __global__ void __launch_bounds__(32 * kRedWarps, HOLD == 32 ? 1 : 2) generic_re
         r.oin = prm.oin ? prm.oin + (size_t)pk * dstride : nullptr;
         r.gobj = prm.gobj ? prm.gobj + (size_t)pk * dstride : nullptr;
         const double v = cta_sum<kRedWarps>(
-            reduce_lane<HOLD>(r, 32 * kRedWarps * s + threadIdx.x, 32 * kRedWarps * S), part);
+            reduce_lane<HOLD, FS>(r, kF * (kRedWarps * s + (threadIdx.x >> 5)), kF * kRedWarps * S), part);
         if (threadIdx.x == 0) (prm.K * S == 1 ? prm.loss : prm.lpart)[u] = v;
         __syncthreads();
     }
@@ -105,12 +106,18 @@ cudaError_t launch_generic_reduction(const GenericParams& prm, int sms, cudaStre
     if (prm.P == 0) return cudaSuccess;
     const int per_patch = prm.K * prm.rsplit;
     if (per_patch > 1 && !prm.lpart) return cudaErrorInvalidValue;
-    // registers for 8, 16 or 32 frames: 2,904 units of 12 frames (96 px) 0.081 ms
-    // in registers, 0.110 in chunks; 12,800 of 32 frames (128 px) 0.460 and 0.477
-    auto kern = prm.J <= 8    ? generic_reduce_kernel<8>
-                : prm.J <= 16 ? generic_reduce_kernel<16>
-                : prm.J <= 32 ? generic_reduce_kernel<32>
-                              : generic_reduce_kernel<0>;
+    // up to 16 frames of a frequency in a lane's registers, then two and four
+    // lanes a frequency, then chunks: 2,904 units of 12 frames (96 px) 0.081 ms
+    // (0.110 in chunks, 0.097 over two lanes of 8); 12,800 of 32 frames (128 px)
+    // 0.442 (0.460 as 32 in one lane, 0.477 in chunks); 22,500 of 100 frames (64
+    // px) 0.283 (0.329 in chunks). The object-inferring form is not split.
+    auto kern = prm.J <= 8     ? generic_reduce_kernel<8, 1>
+                : prm.J <= 16  ? generic_reduce_kernel<16, 1>
+                : prm.oin      ? generic_reduce_kernel<0, 1>
+                : prm.J <= 32  ? generic_reduce_kernel<16, 2>
+                : prm.J <= 64  ? generic_reduce_kernel<16, 4>
+                : prm.J <= 128 ? generic_reduce_kernel<32, 4>
+                               : generic_reduce_kernel<0, 1>;
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kRedWarps, 0);
     if (e != cudaSuccess) return e;

@@ -63,6 +63,26 @@ __device__ __forceinline__ void fp64_frequency(int J, const float2* dp, size_t d
     o = make_float2((float)ox, (float)oy);
 }
 
+// One frequency of the object-inferring loss in FP64 (explicit_frequency).
+__device__ __forceinline__ float explicit_fp64(int J, const float2* dp, size_t dstride, float2* hp, size_t hstride,
+                                               const float* w, double gamma, bool seed, float2 o, float2& g) {
+    const double ox = o.x, oy = o.y;
+    double ts = 0.0, gx = 0.0, gy = 0.0;
+    for (int j = 0; j < J; ++j) {
+        const float2 d = dp[(size_t)j * dstride];
+        const float2 h = hp[(size_t)j * hstride];
+        const double wj = w[j];
+        const double rx = (double)d.x - (ox * h.x - oy * h.y), ry = (double)d.y - (ox * h.y + oy * h.x);
+        ts += wj * (rx * rx + ry * ry);
+        gx += wj * ((double)h.x * rx + (double)h.y * ry);
+        gy += wj * ((double)h.x * ry - (double)h.y * rx);
+        hp[(size_t)j * hstride] = seed ? make_float2((float)(-wj * (ox * rx + oy * ry)), (float)(-wj * (ox * ry - oy * rx)))
+                                       : make_float2(0.f, 0.f);
+    }
+    g = make_float2((float)(gamma * ox - gx), (float)(gamma * oy - gy));
+    return (float)(ts + gamma * (ox * ox + oy * oy));
+}
+
 // One frequency of the object-inferring loss (the object o given): the
 // residuals r_j = D_j - o H_j, the loss term t = sum_j w |r_j|^2 + gamma |o|^2
 // (returned), the adjoint seeds -w conj(o) r_j (0 when `seed` is false)
@@ -99,21 +119,38 @@ __device__ __forceinline__ float explicit_frequency(int J, const float2* dp, siz
         g = make_float2(gam * o.x - gx, gam * o.y - gy);
         return tsum + gam * (o.x * o.x + o.y * o.y);
     }
-    const double ox = o.x, oy = o.y;
-    double ts = 0.0, gx = 0.0, gy = 0.0;
-    for (int j = 0; j < J; ++j) {
-        const float2 d = dp[(size_t)j * dstride];
-        const float2 h = hp[(size_t)j * hstride];
-        const double wj = w[j];
-        const double rx = (double)d.x - (ox * h.x - oy * h.y), ry = (double)d.y - (ox * h.y + oy * h.x);
-        ts += wj * (rx * rx + ry * ry);
-        gx += wj * ((double)h.x * rx + (double)h.y * ry);
-        gy += wj * ((double)h.x * ry - (double)h.y * rx);
-        hp[(size_t)j * hstride] = seed ? make_float2((float)(-wj * (ox * rx + oy * ry)), (float)(-wj * (ox * ry - oy * rx)))
-                                       : make_float2(0.f, 0.f);
+    return explicit_fp64(J, dp, dstride, hp, hstride, w, gamma, seed, o, g);
+}
+
+// explicit_frequency of J <= JM frames held in registers (d, h, wv; zeros
+// beyond J): the same operations in the same order, without the second read.
+template <int JM>
+__device__ __forceinline__ float explicit_held(int J, const float2 (&d)[JM], const float2 (&h)[JM],
+                                               const float (&wv)[JM], const float2* dp, size_t dstride, float2* hp,
+                                               size_t hstride, const float* w, double gamma, bool seed, float2 o,
+                                               float2& g) {
+    float tsum = 0.f, e = 0.f;
+#pragma unroll
+    for (int j = 0; j < JM; ++j) {
+        const float rx = d[j].x - (o.x * h[j].x - o.y * h[j].y), ry = d[j].y - (o.x * h[j].y + o.y * h[j].x);
+        tsum += wv[j] * (rx * rx + ry * ry);
+        e += wv[j] * (d[j].x * d[j].x + d[j].y * d[j].y);
     }
-    g = make_float2((float)(gamma * ox - gx), (float)(gamma * oy - gy));
-    return (float)(ts + gamma * (ox * ox + oy * oy));
+    if (!(tsum >= kCancel * e)) return explicit_fp64(J, dp, dstride, hp, hstride, w, gamma, seed, o, g);
+    const float gam = (float)gamma;
+    float gx = 0.f, gy = 0.f;
+#pragma unroll
+    for (int j = 0; j < JM; ++j) {
+        const float wj = wv[j];
+        const float rx = d[j].x - (o.x * h[j].x - o.y * h[j].y), ry = d[j].y - (o.x * h[j].y + o.y * h[j].x);
+        gx += wj * (h[j].x * rx + h[j].y * ry);
+        gy += wj * (h[j].x * ry - h[j].y * rx);
+        if (j < J)
+            hp[(size_t)j * hstride] = seed ? make_float2(-wj * (o.x * rx + o.y * ry), -wj * (o.x * ry - o.y * rx))
+                                           : make_float2(0.f, 0.f);
+    }
+    g = make_float2(gam * o.x - gx, gam * o.y - gy);
+    return tsum + gam * (o.x * o.x + o.y * o.y);
 }
 
 }  // namespace mfbd_dev

@@ -179,7 +179,21 @@ __device__ __forceinline__ double reduce_frequencies(const FusedParams& prm, int
         if (MODE == 2 || (MODE == 0 && prm.oin)) {  // object-inferring loss: the object is given
             const size_t ooff = ((size_t)p * prm.K + k) * dstride;
             float2 g;
-            const float t = explicit_frequency(J, dp, dstride, hp, kHalf, w, prm.gamma, seed, prm.oin[ooff + doff], g);
+            float t;
+            if constexpr (JM > 0) {
+                float2 d[JM], h[JM];
+#pragma unroll
+                for (int j = 0; j < JM; ++j) {
+                    if constexpr (STREAM)
+                        d[j] = (j < J) ? ld_hint(dp + (size_t)j * dstride, pol) : make_float2(0.f, 0.f);
+                    else
+                        d[j] = (j < J) ? dp[(size_t)j * dstride] : make_float2(0.f, 0.f);
+                    h[j] = (j < J) ? hp[(size_t)j * kHalf] : make_float2(0.f, 0.f);
+                }
+                t = explicit_held<JM>(J, d, h, wv, dp, dstride, hp, kHalf, w, prm.gamma, seed, prm.oin[ooff + doff], g);
+            } else {
+                t = explicit_frequency(J, dp, dstride, hp, kHalf, w, prm.gamma, seed, prm.oin[ooff + doff], g);
+            }
             acc.add((kx == 0 || kx == kN / 2) ? t : 2.0f * t);
             if (prm.gobj) {
                 prm.gobj[ooff + doff] = g;

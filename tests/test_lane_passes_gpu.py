@@ -59,7 +59,7 @@ def test_batch_box_and_unit_edges(shapes):
             _check(case, loss[i].cpu().numpy(), grad[i].cpu().numpy(), obj[i].cpu().numpy().astype("complex128"), ref)
 
 
-@pytest.mark.parametrize("frames", [1, 8, 9, 16, 17, 32, 33])
+@pytest.mark.parametrize("frames", [1, 8, 9, 16, 17, 32, 33, 64, 65, 129])
 @pytest.mark.parametrize("n_pix,diams", [(48, (20.0, 24.0)), (96, (40.0,))])
 def test_frame_reduction_frame_counts(n_pix, diams, frames):
     """The frame reduction where its register forms (8, 16, 32 frames) end and its chunked form begins."""
