@@ -78,8 +78,19 @@ __global__ void __launch_bounds__(32 * kWarps<N>, kMinCtas<N, true, RECOMPUTE>) 
     load_twiddles<N>(tw, threadIdx.x, 32 * kWarps<N>);
     __syncthreads();
     const long long units = (long long)prm.P * prm.K * prm.J;
-    for (long long u = blockIdx.x; u < units; u += gridDim.x)
+    for (long long u = blockIdx.x; u < units; u += gridDim.x) {
+        // the next unit's seed (and phase) from HBM into L2 under this unit: 12,800
+        // units of 128 px 1.038 -> 1.000 ms, 6,750 of 64 px 0.138 -> 0.129; not where
+        // it was slower (96 px 0.130 -> 0.133, 48 px 0.216 -> 0.221, 128 px with the
+        // field kept 0.866 -> 0.892)
+        if (N == 64 || (N == 128 && RECOMPUTE))
+            if (threadIdx.x == 32 * kWarps<N> - 1 && u + gridDim.x < units) {
+                const UnitPtr n = unit_ptr<N>(prm, u + gridDim.x);
+                prefetch_l2(n.h, 8u * N * Geo<N>::NH);
+                if (RECOMPUTE && n.W % 2 == 0) prefetch_l2(n.phi, 4u * n.W * n.W);  // rows of whole 16-byte groups
+            }
         unit_adjoint<N, S, kWarps<N>, RECOMPUTE>(unit_ptr<N>(prm, u), E, E2, prm.es2, tw, w, lane, CtaBar{});
+    }
 }
 
 template <class Kern>

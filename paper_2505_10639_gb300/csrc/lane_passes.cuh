@@ -60,6 +60,11 @@ struct ColumnBits {
     __device__ __forceinline__ bool bit(int b) const { return (w[b >> 5] >> (b & 31)) & 1u; }
 };
 
+// L2 prefetch of `bytes` (a multiple of 16) from a 16-byte aligned address.
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "r"(bytes) : "memory");
+}
+
 // Everything one unit's passes touch.
 struct UnitPtr {
     const float* phi;       // [W][W] box phase
