@@ -36,6 +36,7 @@
 // The pair's loss (the threads' Kahan sums, combined in a fixed order) goes
 // to lpair[p][k]; the CTA that completes a patch's last object (a per-patch
 // counter, reset after use) sums its objects' losses in object order.
+#include "chained.cuh"
 #include "mfbd_internal.h"
 #include "fft_reg.cuh"
 #include "mfbd_device.cuh"
@@ -165,6 +166,8 @@ __global__ void __launch_bounds__(kFT, 1) fused_pair_kernel(const FusedParams pr
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = s_tmem;
+    chain_wait();
+    chain_release();
     auto tmem_row = [&]() {  // this lane's row of the warp's columns
         return tmem_base + ((uint32_t)(32 * ((threadIdx.x >> 5) & 3)) << 16) + (uint32_t)((threadIdx.x >> 7) * 128);
     };
@@ -492,8 +495,7 @@ cudaError_t launch_pairs_es(const FusedParams& prm, int ctas, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(fused_pair_kernel<ES, EXPL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    fused_pair_kernel<ES, EXPL><<<ctas, kFT, smem, s>>>(prm);
-    return cudaGetLastError();
+    return launch_chained(prm.chain, fused_pair_kernel<ES, EXPL>, ctas, kFT, smem, s, prm);
 }
 
 template <int ES>

@@ -2,6 +2,7 @@
 //   phi[u][i]  = c_k sum_m a[u][m] B_k[m][i]          (u = patch*J + frame)
 //   g_a[u][m] (+)= c_k sum_i dL/dphi[u][i] B_k[m][i]
 // Register-tiled SIMT kernels with the operands staged in shared memory.
+#include "chained.cuh"
 #include "mfbd_internal.h"
 
 #include <cstdint>
@@ -188,6 +189,7 @@ __global__ void __launch_bounds__(kGT, 3) grad_gemm_kernel(const GradJob job, in
 
 // grad[e] = sum_k scale_k sum_z part_k[z][e], in a fixed order
 __global__ void __launch_bounds__(256) grad_combine_kernel(const GradParts gp, size_t n, float* __restrict__ grad) {
+    chain_wait();
     for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
         float v = 0.f;
         for (int k = 0; k < gp.K; ++k) {
@@ -266,8 +268,7 @@ cudaError_t launch_grad_combine(const GradParts& gp, int U, int M, float* grad, 
     if (n == 0) return cudaSuccess;
     size_t blocks = (n + 255) / 256;
     if (blocks > 4096) blocks = 4096;
-    grad_combine_kernel<<<(int)blocks, 256, 0, s>>>(gp, n, grad);
-    return cudaGetLastError();
+    return launch_chained(gp.chain, grad_combine_kernel, (int)blocks, 256, 0, s, gp, n, grad);
 }
 
 }  // namespace mfbd_dev

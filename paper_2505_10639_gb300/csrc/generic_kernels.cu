@@ -4,6 +4,7 @@
 #include <algorithm>
 
 #include "mfbd_internal.h"
+#include "chained.cuh"
 #include "frame_reduction.cuh"
 
 namespace mfbd_dev {
@@ -28,6 +29,8 @@ __global__ void __launch_bounds__(32 * kRedWarps, HOLD == 32 ? 1 : 2) generic_re
     const int N = prm.N, half = N * (N / 2 + 1), J = prm.J, S = prm.rsplit;
     const size_t dstride = (size_t)N * prm.spec_ld;
     const long long work = (long long)prm.P * prm.K * S;
+    chain_wait();
+    chain_release();
     for (long long u = blockIdx.x; u < work; u += gridDim.x) {
         const long long pk = u / S;
         const int s = (int)(u - pk * S), k = (int)(pk % prm.K);
@@ -53,6 +56,8 @@ __global__ void __launch_bounds__(32 * kRedWarps, HOLD == 32 ? 1 : 2) generic_re
 
 __global__ void loss_combine_kernel(const double* __restrict__ lpart, int S, double* __restrict__ loss, int P) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    chain_wait();
+    chain_release();
     if (p >= P) return;
     double tot = 0.0;
     for (int i = 0; i < S; ++i) tot += lpart[(size_t)p * S + i];
@@ -123,9 +128,9 @@ cudaError_t launch_generic_reduction(const GenericParams& prm, int sms, cudaStre
     if (e != cudaSuccess) return e;
     long long ctas = (long long)sms * (per_sm > 0 ? per_sm : 1);
     if (ctas > (long long)prm.P * per_patch) ctas = (long long)prm.P * per_patch;
-    kern<<<(int)ctas, 32 * kRedWarps, 0, s>>>(prm);
-    if ((e = cudaGetLastError()) != cudaSuccess || per_patch == 1) return e;
-    return launch_loss_combine(prm.lpart, per_patch, prm.loss, prm.P, s);
+    e = launch_chained(prm.chain, kern, (int)ctas, 32 * kRedWarps, 0, s, prm);
+    if (e != cudaSuccess || per_patch == 1) return e;
+    return launch_loss_combine(prm.lpart, per_patch, prm.loss, prm.P, s, prm.chain);
 }
 
 int generic_reduction_split(int P, int K, int N, int sms) {
@@ -142,10 +147,9 @@ int reduction_split(int P, int K, int N, int sms) {
     return (int)std::min((want + warps - 1) / warps, smax);
 }
 
-cudaError_t launch_loss_combine(const double* lpart, int S, double* loss, int P, cudaStream_t s) {
+cudaError_t launch_loss_combine(const double* lpart, int S, double* loss, int P, cudaStream_t s, bool chain) {
     if (P == 0) return cudaSuccess;
-    loss_combine_kernel<<<(P + 127) / 128, 128, 0, s>>>(lpart, S, loss, P);
-    return cudaGetLastError();
+    return launch_chained(chain, loss_combine_kernel, (P + 127) / 128, 128, 0, s, lpart, S, loss, P);
 }
 
 }  // namespace mfbd_dev

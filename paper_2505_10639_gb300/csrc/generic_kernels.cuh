@@ -7,6 +7,8 @@
 #pragma once
 
 #include <algorithm>
+
+#include "chained.cuh"
 #include "mfbd_internal.h"
 #include "lane_passes.cuh"
 
@@ -60,6 +62,7 @@ __global__ void __launch_bounds__(32 * kWarps<N>, kMinCtas<N, false, false>) gen
     float2* E = tw + Twiddles<N>::kElems;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     load_twiddles<N>(tw, threadIdx.x, 32 * kWarps<N>);
+    chain_wait();  // no chain_release: the reduction, resident early, would run with these CTAs' L1 split
     __syncthreads();
     const long long units = (long long)prm.P * prm.K * prm.J;
     for (long long u = blockIdx.x; u < units; u += gridDim.x)
@@ -76,6 +79,8 @@ __global__ void __launch_bounds__(32 * kWarps<N>, kMinCtas<N, true, RECOMPUTE>) 
     // in L2) so that shared memory holds one exchange buffer
     float2* E2 = RECOMPUTE ? prm.e2scr + (size_t)blockIdx.x * N * prm.es2 : nullptr;
     load_twiddles<N>(tw, threadIdx.x, 32 * kWarps<N>);
+    chain_wait();
+    chain_release();
     __syncthreads();
     const long long units = (long long)prm.P * prm.K * prm.J;
     for (long long u = blockIdx.x; u < units; u += gridDim.x) {
@@ -113,8 +118,7 @@ cudaError_t launch_persistent(Kern kern, int threads, size_t smem, long long uni
     if (e != cudaSuccess) return e;
     if (max_ctas > 0 && ctas > max_ctas) ctas = max_ctas;
     if (ctas > units) ctas = units;
-    kern<<<(int)ctas, threads, smem, s>>>(prm);
-    return cudaGetLastError();
+    return launch_chained(prm.chain, kern, (int)ctas, threads, smem, s, prm);
 }
 
 }  // namespace

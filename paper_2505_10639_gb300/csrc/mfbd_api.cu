@@ -66,6 +66,7 @@ struct mfbd_plan {
     unsigned flags = 0;
     int precision = MFBD_PREC_FP32;
     bool generic = false;       // CTA-per-unit kernels (N != 64, recompute, or on request)
+    bool chain = false;         // the kernels of the call at hand are chained (chain_call)
     bool fused = false;         // mfbd_loss_grad runs the fused per-(patch, object) kernel
     int fused_ctas = 0;         // its CTAs (one per SM)
     float2* d_fscr = nullptr;   // its field slots [fused_ctas][kFusedFrames][N*N/2] (rows N/2..N-1)
@@ -287,6 +288,7 @@ FusedParams fused_params(const mfbd_plan* p, int p0, int np, const void* spectra
     f.K = p->K;
     f.J = p->J;
     f.M = p->M;
+    f.chain = p->chain;
     f.gamma = p->gamma;
     f.weights = p->d_weights;
     f.phi = p->d_phi;
@@ -334,6 +336,21 @@ int set_device(mfbd_plan_t p) {
     return MFBD_OK;
 }
 
+// Whether the kernels of the call at hand are launched with their prologues
+// over their predecessors (chained.cuh). On a stream (whole evaluations, us):
+// 7x7 patches of 128 px 215 -> 198, 11x11 of 96 px 364 -> 355, 15x15 of 64 px
+// with 15 frames 353 -> 343, one patch of 64 px 80 -> 72. Not the fused kernel
+// beyond one pair per CTA (961 patches 875 -> 886), and not under capture: a
+// graph's launches have little latency left to hide (96 px 340 -> 344).
+void chain_call(mfbd_plan_t p, cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        st = cudaStreamCaptureStatusActive;
+    }
+    p->chain = st == cudaStreamCaptureStatusNone && (!p->fused || (long long)p->P * p->K <= p->fused_ctas);
+}
+
 // event pair around one launch when profiling: returns the pair index or -1
 int prof_begin(mfbd_plan_t p, int kind, cudaStream_t s) {
     if (p->ev.empty() || p->ev_used * 2 >= (int)p->ev.size()) return -1;
@@ -370,7 +387,7 @@ int run_phase(mfbd_plan_t p, const float* coeffs, cudaStream_t s, int p0, int np
         cudaError_t e = launch_split_coeffs(coeffs, U, p->M, p->obj[0].tc_planes, p->d_acoef, s);
         if (e == cudaSuccess)
             e = launch_phase_mma(p->d_acoef, U, p->M, p->K, bt, npix, p->obj[0].tc_planes, scale, out, p->d_err,
-                                 p->sms, s);
+                                 p->sms, p->chain, s);
         for (int k = 0; k < p->K && e == cudaSuccess; ++k)  // phi_kj = c_k B_k a_j + theta_kj
             if (p->obj[k].d_div) e = launch_add_diversity(out[k], p->obj[k].d_div, U, p->J, npix[k], p->sms, s);
         prof_end(p, pi, s, 2 + ndiv);
@@ -413,6 +430,7 @@ int run_grad(mfbd_plan_t p, float* grad, cudaStream_t s, int p0, int np) {
     }
     GradParts gp{};
     gp.K = p->K;
+    gp.chain = p->chain;
     for (int k = 0; k < p->K; ++k) {
         const ObjectData& o = p->obj[k];
         job.gphi[k] = p->d_gphi + o.phi_off + (size_t)p0 * p->J * o.W * o.W;
@@ -434,6 +452,7 @@ int run_grad(mfbd_plan_t p, float* grad, cudaStream_t s, int p0, int np) {
         mj.M = p->M;
         mj.row0 = p0 * p->J;
         mj.err = p->d_err;
+        mj.chain = p->chain;
         for (int k = 0; k < p->K; ++k) {
             mj.gmap[k] = &p->obj[k].gmap;
             mj.bpl[k] = p->obj[k].d_gbasis_tc;
@@ -474,6 +493,7 @@ int run_generic(mfbd_plan_t p, int stages, const void* spectra, double* loss, vo
     g.gphi = p->d_gphi;
     const bool otf_only = (stages & ST_OTF_ONLY) != 0;
     g.otf_only = otf_only;
+    g.chain = p->chain;
     g.gscr = otf_only ? gscr : p->d_gscr;
     g.pscr = otf_only ? nullptr : p->d_pscr;
     g.spectra = static_cast<const float2*>(spectra);
@@ -1188,6 +1208,7 @@ int mfbd_forward(mfbd_plan_t p, const float* coeffs, const void* spectra, double
     if (!coeffs || !spectra || !loss) return fail(MFBD_ERR_INVALID_ARG, "coeffs, spectra and loss are required");
     if ((st = set_device(p))) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    chain_call(p, s);
     if ((st = run_phase(p, coeffs, s, 0, p->P))) return st;
     if ((st = run_fused(p, ST_FWD | ST_RED, spectra, loss, object, p->d_gscr, s, 0, p->P))) return st;
     p->have_forward = true;
@@ -1202,6 +1223,7 @@ int mfbd_backward(mfbd_plan_t p, float* grad, void* stream) {
     if (!grad) return fail(MFBD_ERR_INVALID_ARG, "grad is NULL");
     if ((st = set_device(p))) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    chain_call(p, s);
     if ((st = run_fused(p, ST_ADJ, nullptr, nullptr, nullptr, p->d_gscr, s, 0, p->P))) return st;
     return run_grad(p, grad, s, 0, p->P);
 }
@@ -1215,6 +1237,7 @@ int mfbd_loss_grad(mfbd_plan_t p, const float* coeffs, const void* spectra, doub
         return fail(MFBD_ERR_INVALID_ARG, "coeffs, spectra, loss and grad are required");
     if ((st = set_device(p))) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    chain_call(p, s);
     if ((st = run_phase(p, coeffs, s, 0, p->P))) return st;
     if (p->fused) {  // one launch; nothing is kept for mfbd_backward
         p->have_forward = false;
@@ -1236,6 +1259,7 @@ int mfbd_loss_grad_explicit(mfbd_plan_t p, const float* coeffs, const void* spec
         return fail(MFBD_ERR_INVALID_ARG, "coeffs, spectra, object, loss and grad are required");
     if ((st = set_device(p))) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    chain_call(p, s);
     p->have_forward = false;  // the seeds will belong to the given objects
     if ((st = run_phase(p, coeffs, s, 0, p->P))) return st;
     p->x_oin = object;
@@ -1274,6 +1298,7 @@ int mfbd_loss_grad_host(mfbd_plan_t p, const float* coeffs, const void* spectra,
     auto& h = p->host;
     const size_t sp = spectrum_patch_bytes(p), op = object_patch_bytes(p);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    p->chain = false;  // copies and events stand between the kernels
     cudaError_t e = cudaSuccess;
 #define MFBD_HOST_TRY(call)                        \
     if ((e = (call)) != cudaSuccess) {             \
@@ -1337,6 +1362,7 @@ int mfbd_otf(mfbd_plan_t p, const float* coeffs, void* otf, void* stream) {
     if (!coeffs || !otf) return fail(MFBD_ERR_INVALID_ARG, "coeffs and otf are required");
     if ((st = set_device(p))) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    chain_call(p, s);
     p->have_forward = false;  // the phases now belong to these coefficients
     if ((st = run_phase(p, coeffs, s, 0, p->P))) return st;
     return run_fused(p, ST_FWD | ST_OTF_ONLY, nullptr, nullptr, nullptr, static_cast<float2*>(otf), s, 0, p->P);

@@ -40,6 +40,7 @@ struct FusedParams {
     float2* pscr;             // [P][K][J][N x N]: field p = F P, stored [x][y] (null: not kept)
     float2* uscr;             // [P][K][J][ustride]: pupil phasors exp(i phi) on the box (null: not kept)
     int ustride;              // complex elements per unit in uscr (>= W_k^2 for every object)
+    bool chain;               // launched with its prologue over its predecessor (chained.cuh)
     const float2* spectra;    // D
     int spec_ld;              // row stride of D and O in complex elements (33 or 64)
     double* loss;             // [P]
@@ -105,7 +106,8 @@ cudaError_t launch_split_coeffs(const float* a, int U, int M, int planes, uint16
 // One launch for the K objects: bt[k] the basis planes of object k (npix[k]
 // pixels), phase[k] its [U][npix[k]] output, scaled by scale[k].
 cudaError_t launch_phase_mma(const uint16_t* at, int U, int M, int K, const uint16_t* const* bt, const int* npix,
-                             int planes, const float* scale, float* const* phase, int* err, int sms, cudaStream_t s);
+                             int planes, const float* scale, float* const* phase, int* err, int sms, bool chain,
+                             cudaStream_t s);
 
 // Modal adjoint, one launch for all objects: part_k[z][u][m] = sum over
 // pixel chunk z of object k of gphi_k[u][i] basis_k[m][i]. grad_layout picks
@@ -142,6 +144,7 @@ struct GradMmaJob {
     int npix[kMaxObjects];
     int chunk[kMaxObjects];
     int* err;                          // set to 1 when a wait gives up
+    bool chain;
 };
 int grad_mma_ring(int M);
 size_t grad_mma_smem(int M, int ring);
@@ -157,6 +160,7 @@ struct GradParts {
     int splits[kMaxObjects];
     float scale[kMaxObjects];
     const float* part[kMaxObjects];
+    bool chain;
 };
 cudaError_t launch_grad_combine(const GradParts& gp, int U, int M, float* grad, cudaStream_t s);
 
@@ -192,6 +196,7 @@ struct GenericParams {
     int e2_ctas;            // CTAs e2scr has room for
     int rsplit;             // CTAs that share a (patch, object) of the frame reduction
     double* lpart;          // K rsplit > 1: their losses [P][K][rsplit]
+    bool chain;             // launched with their prologues over their predecessors (chained.cuh)
     bool otf_only;          // gscr is the caller's OTF: also written outside the support
     const float2* oin;      // object-inferring loss: the given objects [P][K][N][spec_ld], else null
     float2* gobj;           // with oin: dL/dconj(O) [P][K][N][spec_ld], or null
@@ -220,7 +225,7 @@ int reduction_split(int P, int K, int N, int sms);
 // they are few. Fixed by a plan like reduction_split.
 int generic_reduction_split(int P, int K, int N, int sms);
 // loss[p] = sum over s < S of lpart[p][s], in order.
-cudaError_t launch_loss_combine(const double* lpart, int S, double* loss, int P, cudaStream_t s);
+cudaError_t launch_loss_combine(const double* lpart, int S, double* loss, int P, cudaStream_t s, bool chain = false);
 
 // ----------------------------------------- data front and back end of a field
 struct FrontParams {

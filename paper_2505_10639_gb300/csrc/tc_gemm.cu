@@ -22,6 +22,7 @@
 // eight epilogue warps drain tile n - 1 from the other accumulator and the
 // copy of tile n + 1 is in flight. In the epilogue a lane holds one pixel, so each store
 // instruction writes 32 consecutive pixels of one unit's phase row.
+#include "chained.cuh"
 #include "mfbd_internal.h"
 #include "umma.cuh"
 
@@ -81,6 +82,7 @@ __device__ __forceinline__ void bf16_split3(float x, uint32_t& b0, uint32_t& b1,
 // [n_tiles][planes][128 units x Mp modes]; one thread per (unit, 8 modes).
 __global__ void __launch_bounds__(256) split_coeffs_kernel(const float* __restrict__ a, int U, int M, int Mp,
                                                            int planes, uint16_t* __restrict__ out) {
+    chain_release();
     const int kcs = Mp / 8;
     const int n_tiles = (U + kTile - 1) / kTile;
     const long long total = (long long)n_tiles * kTile * kcs;
@@ -152,10 +154,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_mma_kernel(const PhaseMma
     auto unit_src = [&](int n) { return q.at + (size_t)(g0 + n * gs) * planes * kTile * Mp; };
 
     copy_tile(sP, q.bt[k] + (size_t)it * planes * kTile * Mp);
-    if (n_tiles > 0) copy_tile(sU[0], unit_src(0));
-    cp_async_commit();
-    if (n_tiles > 1) copy_tile(sU[1], unit_src(1));
-    cp_async_commit();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_base_s)),
                      "r"(2 * kTile));
@@ -168,6 +166,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) phase_mma_kernel(const PhaseMma
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    chain_wait();  // the coefficient planes; the phases may be overwritten
+    chain_release();
+    if (n_tiles > 0) copy_tile(sU[0], unit_src(0));
+    cp_async_commit();
+    if (n_tiles > 1) copy_tile(sU[1], unit_src(1));
+    cp_async_commit();
     const uint32_t tmem = tmem_base_s;
     const uint32_t idesc = instr_desc_bf16(kTile, kTile);
     const int lq = warp & 3, ch = warp >> 2;  // TMEM lane quarter (pixels), unit-column half
@@ -260,7 +264,8 @@ cudaError_t launch_split_coeffs(const float* a, int U, int M, int planes, uint16
 }
 
 cudaError_t launch_phase_mma(const uint16_t* at, int U, int M, int K, const uint16_t* const* bt, const int* npix,
-                             int planes, const float* scale, float* const* phase, int* err, int sms, cudaStream_t s) {
+                             int planes, const float* scale, float* const* phase, int* err, int sms, bool chain,
+                             cudaStream_t s) {
     if (U == 0 || K == 0) return cudaSuccess;
     if (K > kMaxObjects) return cudaErrorInvalidValue;
     PhaseMmaParams q;
@@ -306,8 +311,7 @@ cudaError_t launch_phase_mma(const uint16_t* at, int U, int M, int K, const uint
     q.groups = groups;
     q.cta0[0] = 0;
     for (int k = 0; k < K; ++k) q.cta0[k + 1] = q.cta0[k] + groups * q.n_itiles[k];
-    phase_mma_kernel<<<q.cta0[K], kTcThreads, smem, s>>>(q);
-    return cudaGetLastError();
+    return launch_chained(chain, phase_mma_kernel, q.cta0[K], kTcThreads, smem, s, q);
 }
 
 }  // namespace mfbd_dev

@@ -30,6 +30,7 @@
 // and a CTA-wide abort flag that ends the other roles' loops; the CTA then
 // waits (bounded) for its copies and MMAs in flight and frees its tensor
 // memory before it returns.
+#include "chained.cuh"
 #include "mfbd_internal.h"
 #include "tma.cuh"
 #include "umma.cuh"
@@ -177,6 +178,8 @@ __global__ void __launch_bounds__(kGThreads, 1) grad_mma_kernel(const __grid_con
     __syncthreads();
     umma::fence_after_sync();
     const uint32_t tmem = tmem_s;
+    chain_wait();  // dL/dphi; the partial sums may be overwritten
+    chain_release();
 
     if (warp == kGConv) {
         // ------------------------------------------------------------ producer
@@ -470,8 +473,7 @@ cudaError_t launch_grad_mma(const GradMmaJob& job, int sms, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(grad_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int grid = (int)std::min<long long>(items, sms);
-    grad_mma_kernel<<<grid, kGThreads, smem, s>>>(q);
-    return cudaGetLastError();
+    return launch_chained(job.chain, grad_mma_kernel, grid, kGThreads, smem, s, q);
 }
 
 }  // namespace mfbd_dev
