@@ -53,6 +53,7 @@ struct FusedParams {
     double* lpair;            // fused kernel: per (patch, object) losses [P][K]
     int* lcnt;                // fused kernel: per patch, the objects done [P] (0 between calls)
     int* fticket;             // fused kernel: [0] next-pair ticket, [1] CTAs done (0 between calls)
+    int csize;                // spread kernel: CTAs per pair
     int korder[kMaxObjects];  // fused kernel: objects in the order their pairs are dealt
     ObjParams obj[kMaxObjects];
 };
@@ -86,6 +87,13 @@ size_t fused_pair_smem(int es);
 bool fused_pair_supported(int J, int es);
 int fused_pair_ctas_per_sm(int es);
 cudaError_t launch_fused_pairs(const FusedParams& prm, int es, int ctas, cudaStream_t s);
+
+// The same with a cluster of prm.csize CTAs per pair, for few pairs
+// (spread_kernels.cu); gscr holds the plan's per-unit OTF / seed buffers, lpair
+// P x K x csize losses. spread_cluster: the cluster size for a plan, 0 where the
+// fused kernel is the better one or the clusters do not fit.
+int spread_cluster(int P, int K, int J, int max_box);
+cudaError_t launch_spread_pairs(const FusedParams& prm, cudaStream_t s);
 
 // phase[u][i] += div[u mod J][i] for U units (U a multiple of J): the
 // known diversity phases of the J frames added to every patch's phases.
