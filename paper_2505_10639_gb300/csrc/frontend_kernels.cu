@@ -2,13 +2,12 @@
 // apodization"): the data spectra of every patch and frame from the frames,
 // and the mosaic of the patch objects.
 //
-// Spectra: one CTA per unit (patch, object, frame), persistent. The patch is
-// staged in shared memory by coalesced row loads; its mean is subtracted,
-// the modified Hanning window w[y] w[x] applied and the mean added back; rows y and y + N/2 are transformed as one complex line
-// and split into two half spectra, then the half-spectrum columns (columns
-// 0 and N/2, real after the row transforms, packed as one line) are
-// transformed along y: the unnormalised 2-D DFT of the apodised patch,
-// kx <= N/2.
+// Spectra: one CTA per unit (patch, object, frame), persistent. The patch's
+// mean is subtracted, the modified Hanning window w[y] w[x] applied and the
+// mean added back; rows y and y + N/2 are transformed as one complex line and
+// split into two half spectra, then the half-spectrum columns (columns 0 and
+// N/2, real after the row transforms, packed as one line) are transformed
+// along y: the unnormalised 2-D DFT of the apodised patch, kx <= N/2.
 //
 // Mosaic: (1) per (patch, object) the inverse 2-D DFT of the object's half
 // spectrum, normalised by 1/N^2: columns along ky (0 and N/2 packed, both
@@ -34,6 +33,7 @@
 // cosf.
 #include "mfbd_internal.h"
 #include "tma.cuh"
+#include "lane_passes.cuh"
 #include "line_fft.cuh"
 
 #include <cmath>
@@ -59,113 +59,158 @@ __device__ void window_to_smem(float* w, int n, int border) {
     }
 }
 
+template <class Kern>
+cudaError_t launch_persistent_front(Kern kern, int threads, size_t smem, long long work, int sms, const FrontParams& prm,
+                                    cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    long long ctas = (long long)sms * per_sm;
+    if (ctas > work) ctas = work;
+    kern<<<(int)ctas, threads, smem, s>>>(prm);
+    return cudaGetLastError();
+}
+
+// Spectra from frames, any patch size and alignment: one CTA of N / 16 warps
+// per unit, persistent, lines of eight lanes (lane8.cuh) as in the passes of the
+// larger sizes: rows y and y + N/2 of the apodised patch as one complex line,
+// then the half-spectrum columns, the two rows' half spectra split on load (line
+// 0 packs the real columns 0 and N/2). The patch is read once, into the
+// registers that the row transforms start from; its mean comes from FP32 sums
+// per thread (fixed order) combined in FP64.
+//   HBM is the floor (frames in, spectra out); what bounds it is the latency
+// of the patch's loads and the exchanges at 16 - 18 warps per SM. With two or
+// four lanes per line, whole lines in registers and the patch staged in shared
+// memory it took, for 20 frames of two objects, 258 us at 48 px (961
+// patches), 212 us at 64 px (961, stride 29), 608 us at 96 px (441) and 250 us
+// at 128 px (225); now 131, 190, 234 and 205 us, 2.1 - 2.5 TB/s. A field too
+// small to fill the chip takes the same time either way (18.5 us, 9 patches).
 template <int N>
-__global__ void __launch_bounds__(FrontCta<N>::THREADS) spectra_kernel(const FrontParams prm) {
-    constexpr int S = Geo<N>::S, L = Geo<N>::L, NH = Geo<N>::NH, LINES = FrontCta<N>::LINES;
-    constexpr int T = FrontCta<N>::THREADS;
+constexpr int kFrontMinCtas = N == 128 ? 2 : N == 96 ? 4 : N == 64 ? 6 : 9;
+
+template <int N>
+__global__ void __launch_bounds__(2 * N, kFrontMinCtas<N>) spectra_kernel(const FrontParams prm) {
+    using lane8::Geo;
+    constexpr int R = Geo<N>::R, M2 = Geo<N>::M2, NH = Geo<N>::NH, S = Geo<N>::S_HALF, W = N / 16;
+    constexpr int kTasks = 2;  // groups of four lines per warp and pass
     extern __shared__ __align__(16) unsigned char fsm[];
-    float* win = reinterpret_cast<float*>(fsm);                     // [N]
-    double* red = reinterpret_cast<double*>(fsm + 16 * ((N * 4 + 15) / 16));  // [THREADS / 32]
-    float2* E = reinterpret_cast<float2*>(fsm + 16 * ((N * 4 + 15) / 16) + 16 * 8);
-    float* Ef = reinterpret_cast<float*>(E);
-    const int es = prm.es;
-    const int t = threadIdx.x, sub = t % S, li = t / S;
-    window_to_smem(win, N, prm.border);  // read after the first barrier below
+    float2* table = reinterpret_cast<float2*>(fsm);
+    float2* E = table + lane8::Twiddles<N>::kElems;
+    __shared__ float win[N];
+    __shared__ double red[W];
+    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+    lane8::load_twiddles<N>(table, t, 32 * W);
+    window_to_smem(win, N, prm.border);
+    const lanepass::RowLanes rl(lane);
+    const lanepass::ColLanes cl(lane);
     const long long units = (long long)prm.P * prm.K * prm.J;
     for (long long u = blockIdx.x; u < units; u += gridDim.x) {
         const int j = (int)(u % prm.J);
         const long long pk = u / prm.J;
-        const int k = (int)(pk % prm.K);
-        const int p = (int)(pk / prm.K);
+        const int k = (int)(pk % prm.K), p = (int)(pk / prm.K);
         const int y0 = (p / prm.nx) * prm.stride, x0 = (p % prm.nx) * prm.stride;
         const float* F = prm.frames + ((size_t)k * prm.J + j) * prm.H * prm.Wimg + (size_t)y0 * prm.Wimg + x0;
-        // the patch into shared memory (coalesced rows; float rows 2 es
-        // apart, in the exchange buffer) and its mean
-        __syncthreads();  // the previous unit's column pass has read E
-        // per-thread FP32 partial sums over four interleaved accumulators
-        // (fixed order), combined across the CTA in FP64
-        constexpr int kPer = N * N / T;
+        float2 v[kTasks][R];
         float part[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            const int e = t + i * T;
-            const int y = e / N, x = e - y * N;
-            const float v = F[(size_t)y * prm.Wimg + x];
-            Ef[(size_t)y * 2 * es + x] = v;
-            part[i & 3] += v;
+        for (int g = 0; g < kTasks; ++g) {
+            const float* r0 = F + (size_t)(4 * (w + W * g) + rl.p) * prm.Wimg + rl.t;
+            const float* r1 = r0 + (size_t)(N / 2) * prm.Wimg;
+#pragma unroll
+            for (int e = 0; e < R; ++e) v[g][e] = make_float2(r0[8 * e], r1[8 * e]);
         }
+#pragma unroll
+        for (int g = 0; g < kTasks; ++g)
+#pragma unroll
+            for (int e = 0; e < R; ++e) {
+                part[2 * (e & 1)] += v[g][e].x;
+                part[2 * (e & 1) + 1] += v[g][e].y;
+            }
         double acc = ((double)part[0] + (double)part[1]) + ((double)part[2] + (double)part[3]);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if ((t & 31) == 0) red[t >> 5] = acc;
-        __syncthreads();
+        if (lane == 0) red[w] = acc;
+        __syncthreads();  // the sums; and the previous unit's columns are read
         double tot = 0.0;
-        for (int w = 0; w < T / 32; ++w) tot += red[w];
+        for (int i = 0; i < W; ++i) tot += red[i];
         const float m = (float)(tot / (N * N));
-        // rows y and y + N/2 of the apodised patch as one complex line; the
-        // line's lanes read both rows before any of them writes the two half
-        // spectra over them
-        // (every lane of a warp runs every round, inactive ones on zeros, so
-        // that the warp-wide __syncwarp and shuffles see all lanes)
-        for (int y0 = 0; y0 < N / 2; y0 += LINES) {
-            const int y = y0 + li;
-            const bool act = y < N / 2;
-            float2 v[L];
+        {
+            const lane8::LaneTwiddles<N> tw(table, rl.t);
 #pragma unroll
-            for (int n = 0; n < L; ++n) {
-                const int x = S * n + sub;
-                float a = 0.f, b = 0.f;
-                if (act) {
-                    a = (Ef[(size_t)y * 2 * es + x] - m) * win[y] * win[x] + m;
-                    b = (Ef[(size_t)(y + N / 2) * 2 * es + x] - m) * win[y + N / 2] * win[x] + m;
+            for (int g = 0; g < kTasks; ++g) {
+                const int i = 4 * (w + W * g) + rl.p;
+                const lane8::RowLine<N, S> ln{E + i * S};
+                const float wy0 = win[i], wy1 = win[i + N / 2];
+                float2 z[8 * M2];
+#pragma unroll
+                for (int e = 0; e < R; ++e) {
+                    const float wx = win[rl.t + 8 * e];
+                    v[g][e] = make_float2((v[g][e].x - m) * wy0 * wx + m, (v[g][e].y - m) * wy1 * wx + m);
                 }
-                v[n] = make_float2(a, b);
+                lane8::strided_to_blocked<N>(ln, v[g], z, tw, rl.t);
+                __syncwarp();
+#pragma unroll
+                for (int q = 0; q < M2; ++q)
+                    if (R % 8 == 0 || rl.t + 8 * q < R)
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) {
+                            const int kx = rl.t + 8 * q + R * c;  // elements N/2.. in row i + N/2
+                            E[(c < 4 ? i : i + N / 2) * S + (c < 4 ? kx : kx - N / 2)] = z[8 * q + c];
+                        }
             }
-            line_fft<N, -1>(v, sub);
-            __syncwarp();
-            fftreg::static_for<0, L>([&](auto kk) {
-                constexpr int kq = decltype(kk)::value;
-                const float2 pc = conj_partner<N, kq>(v);
-                const int kx = sub * L + kq;
-                if (act && kx <= N / 2) {
-                    const float2 ra = cscale(cadd(v[kq], pc), 0.5f);
-                    const float2 d = cscale(csub(v[kq], pc), 0.5f);
-                    E[y * es + kx] = ra;
-                    E[(y + N / 2) * es + kx] = make_float2(d.y, -d.x);
-                }
-            });
         }
         __syncthreads();
-        // columns kx = 1 .. N/2 - 1; line 0 packs the real columns 0 and N/2
         float2* D = prm.spectra + (size_t)u * N * NH;
-        for (int l0 = 0; l0 < N / 2; l0 += LINES) {
-            const int kx = l0 + li;
-            const bool act = kx < N / 2;
-            float2 v[L];
+        const lane8::LaneTwiddles<N> tw(table, cl.t);
+#pragma unroll 1
+        for (int g = 0; g < kTasks; ++g) {
+            const int kx = 4 * (w + W * g) + cl.c;
+            const lane8::ColLine<N, S> ln{E + kx, kx ? N / 2 - 2 * kx : 0};
+            float2 a[R], z[8 * M2];
 #pragma unroll
-            for (int n = 0; n < L; ++n) {
-                const int ky = S * n + sub;
-                v[n] = !act ? make_float2(0.f, 0.f)
-                            : kx == 0 ? make_float2(E[ky * es].x, E[ky * es + N / 2].x) : E[ky * es + kx];
+            for (int e = 0; e < R / 2; ++e) {
+                const float2 b = ln.block(e)[cl.t * S], c = ln.block(e + R / 2)[cl.t * S];
+                a[e] = kx ? make_float2(0.5f * (b.x + c.x), 0.5f * (b.y - c.y)) : make_float2(b.x, c.x);
+                a[e + R / 2] = kx ? make_float2(0.5f * (b.y + c.y), 0.5f * (c.x - b.x)) : make_float2(b.y, c.y);
             }
-            line_fft<N, -1>(v, sub);
-            fftreg::static_for<0, L>([&](auto kk) {
-                constexpr int kq = decltype(kk)::value;
-                const float2 pc = conj_partner<N, kq>(v);
-                const int ky = sub * L + kq;
-                if (!act) {
-                } else if (kx > 0) {
-                    D[ky * NH + kx] = v[kq];
-                } else {
-                    const float2 d0 = cscale(cadd(v[kq], pc), 0.5f);
-                    const float2 d = cscale(csub(v[kq], pc), 0.5f);
-                    D[ky * NH] = d0;
-                    D[ky * NH + N / 2] = make_float2(d.y, -d.x);
-                }
-            });
+            lane8::strided_to_blocked<N>(ln, a, z, tw, cl.t);
+            if (w == 0 && g == 0) {  // the warp of line 0 splits its packed columns through the line's storage
+                __syncwarp();
+                if (kx == 0)
+#pragma unroll
+                    for (int q = 0; q < M2; ++q)
+                        if (R % 8 == 0 || cl.t + 8 * q < R)
+#pragma unroll
+                            for (int c = 0; c < 8; ++c) E[(cl.t + 8 * q + R * c) * S] = z[8 * q + c];
+                __syncwarp();
+                if (kx == 0)
+#pragma unroll
+                    for (int q = 0; q < M2; ++q)
+                        if (R % 8 == 0 || cl.t + 8 * q < R)
+#pragma unroll
+                            for (int c = 0; c < 8; ++c) {
+                                const int ky = cl.t + 8 * q + R * c;
+                                const float2 x = z[8 * q + c], y = E[(ky ? N - ky : 0) * S];
+                                D[ky * NH + N / 2] = make_float2(0.5f * (x.y + y.y), 0.5f * (y.x - x.x));
+                                z[8 * q + c] = make_float2(0.5f * (x.x + y.x), 0.5f * (x.y - y.y));
+                            }
+            }
+#pragma unroll
+            for (int q = 0; q < M2; ++q)
+                if (R % 8 == 0 || cl.t + 8 * q < R)
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) D[(cl.t + 8 * q + R * c) * NH + kx] = z[8 * q + c];
         }
-        __syncthreads();
     }
+}
+
+template <int N>
+cudaError_t launch_spectra_plain(const FrontParams& prm, long long units, int sms, cudaStream_t s) {
+    const size_t smem = (lane8::Twiddles<N>::kElems + (size_t)N * lane8::Geo<N>::S_HALF) * sizeof(float2);
+    return launch_persistent_front(spectra_kernel<N>, 2 * N, smem, units, sms, prm, s);
 }
 
 constexpr int kTmaBoxCols = 32;                            // 128 bytes of float: the swizzle span
@@ -455,24 +500,7 @@ __global__ void __launch_bounds__(256) filter_kernel(const FilterParams prm) {
     }
 }
 
-template <class Kern>
-cudaError_t launch_persistent_front(Kern kern, int threads, size_t smem, long long work, int sms, const FrontParams& prm,
-                                    cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    long long ctas = (long long)sms * per_sm;
-    if (ctas > work) ctas = work;
-    kern<<<(int)ctas, threads, smem, s>>>(prm);
-    return cudaGetLastError();
-}
-
 }  // namespace
-
-size_t front_smem(int N, int es) { return (size_t)16 * ((N * 4 + 15) / 16) + 16 * 8 + (size_t)N * es * sizeof(float2); }
 
 namespace tma {
 
@@ -535,12 +563,11 @@ cudaError_t launch_spectra_from_frames(const FrontParams& prm, int sms, cudaStre
             return cudaGetLastError();
         }
     }
-    const size_t smem = front_smem(prm.N, prm.es);
     switch (prm.N) {
-        case 48: return launch_persistent_front(spectra_kernel<48>, FrontCta<48>::THREADS, smem, units, sms, prm, s);
-        case 64: return launch_persistent_front(spectra_kernel<64>, FrontCta<64>::THREADS, smem, units, sms, prm, s);
-        case 96: return launch_persistent_front(spectra_kernel<96>, FrontCta<96>::THREADS, smem, units, sms, prm, s);
-        case 128: return launch_persistent_front(spectra_kernel<128>, FrontCta<128>::THREADS, smem, units, sms, prm, s);
+        case 48: return launch_spectra_plain<48>(prm, units, sms, s);
+        case 64: return launch_spectra_plain<64>(prm, units, sms, s);
+        case 96: return launch_spectra_plain<96>(prm, units, sms, s);
+        case 128: return launch_spectra_plain<128>(prm, units, sms, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -270,7 +270,6 @@ struct LsFilterParams {
 };
 size_t ls_filter_smem(int N);
 cudaError_t launch_ls_filter(const LsFilterParams& prm, int sms, cudaStream_t s);
-size_t front_smem(int N, int es);
 // Spectra from frames; 64 px patches on 16-byte column boundaries take the
 // TMA-staged kernel (spectra_tma_eligible), the rest the plain one.
 bool spectra_tma_eligible(const FrontParams& prm);

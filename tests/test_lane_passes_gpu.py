@@ -90,3 +90,30 @@ def test_dictionary_units_beyond_one_wave(atoms):
         assert np.array_equal(loss[2 * r:2 * r + 2], one[0])
         assert np.array_equal(go[2 * r:2 * r + 2], one[1]) and np.array_equal(ga[2 * r:2 * r + 2], one[2])
     check_dict(0, *one, oracle_dict(tuple(case), 0))
+
+
+@pytest.mark.parametrize("n,h,w,overlap,border,frames", [
+    (48, 131, 140, 17, 9, 90),    # more units than one wave of the persistent grid at every size, strides and
+    (64, 167, 201, 29, 13, 60),   # widths that are no multiples of four, and a remainder
+    (96, 203, 299, 53, 1, 40),
+    (128, 261, 325, 67, 24, 20),
+])
+def test_spectra_beyond_one_wave(n, h, w, overlap, border, frames):
+    """Data spectra of any size and alignment; 1e-5 relative (max-norm), as for the other spectra."""
+    import numpy as np
+    import torch
+
+    from oracle import mfbd as omfbd
+    from oracle import patches as opatches
+    from paper_2505_10639_gb300.mfbd import Plan
+    g = np.random.default_rng(n)
+    data = (1.0 + 0.1 * g.standard_normal((2, frames, h, w))).astype(np.float32)
+    grid = opatches.patch_grid(h, w, n, overlap)
+    plan = Plan(n, len(grid), [0.4 * n, 0.3 * n], [6563.0, 6563.0 * 4 / 3], frames, 8, gamma=1e-3)
+    units = len(grid) * 2 * frames
+    assert units > 152 * (2 if n == 128 else 4)
+    d = plan.spectra_from_frames(torch.from_numpy(data).cuda(), overlap, border).cpu().numpy()
+    plan.check()
+    ref = omfbd.half_spectrum(opatches.spectra_from_frames(data.astype(np.float64), n, overlap, border))
+    err = np.abs(d - ref).max() / np.abs(ref).max()
+    assert err <= 1e-5, err
