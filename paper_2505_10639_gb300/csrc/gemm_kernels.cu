@@ -13,68 +13,108 @@ namespace {
 
 // ---------------------------------------------------------------- GEMMs
 
+// 4-byte copy into shared memory in the background, zeros where !live (src is
+// then not read).
+__device__ __forceinline__ void copy_async4(float* dst, const float* src, bool live) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(live ? 4 : 0)
+                 : "memory");
+}
+
 // phase[u][i] = scale * sum_m a[u][m] basis[m][i]: 128 x 128 output tile per
 // CTA of 256 threads, 8 x 8 per thread (two 4 x 4 quadrants 64 apart, so
 // that the stores of a row are contiguous across threads), the modes in
-// chunks of 16 staged in shared memory (rows padded to 132 floats).
-constexpr int kPT = 128, kPK = 16, kPS = kPT + 4;
+// steps of 8 copied into shared memory three steps ahead (rows padded to 132
+// floats; one barrier a step). The products run as paired FP32 FMAs, a
+// rounding each as fmaf gives, summed over the modes in order: a pair (a0, a1)
+// of rows times a pair (b0, b1) of pixels and times (b1, b0) gives the 2 x 2
+// block's diagonals, so that neither operand needs its values doubled.
+//   The FMA pipe is the floor: 80 us for 22,500 x 1,024 phases of 135 modes.
+// Those took 179 us with scalar FMAs and one buffer of 16 modes, 175 us with
+// paired FMAs and the next 8 modes loaded into registers (the loads' latency
+// was the largest stall), 152 us with this; 1,408 tiles are 4.6 waves.
+constexpr int kPT = 128, kPK = 8, kPS = kPT + 4, kPStages = 4;
 
 __global__ void __launch_bounds__(256, 2) phase_gemm_kernel(const float* __restrict__ a, int U, int M,
                                                             const float* __restrict__ basis, int npix, float scale,
                                                             float* __restrict__ out, int vec_store) {
-    __shared__ __align__(16) float As[kPK][kPS];  // [m][u]
-    __shared__ __align__(16) float Bs[kPK][kPS];  // [m][i]
+    __shared__ __align__(16) float As[kPStages][kPK][kPS];  // [m][u]
+    __shared__ __align__(16) float Bs[kPStages][kPK][kPS];  // [m][i]
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int u0 = blockIdx.y * kPT, i0 = blockIdx.x * kPT;
-    float acc[8][8];
+    const int am = threadIdx.x & (kPK - 1), au = threadIdx.x / kPK;  // a: 8 consecutive modes of one row
+    const int bi = threadIdx.x & (kPT - 1), bm = threadIdx.x / kPT;  // basis: 128 consecutive pixels of one mode
+    const int steps = (M + kPK - 1) / kPK;
+    auto fetch = [&](int step) {
+        const int m0 = step * kPK, buf = step % kPStages;
+        if (step < steps) {
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
-#pragma unroll
-        for (int c = 0; c < 8; ++c) acc[r][c] = 0.f;
-    for (int m0 = 0; m0 < M; m0 += kPK) {
-#pragma unroll
-        for (int t = 0; t < kPT * kPK / 256; ++t) {
-            const int idx = threadIdx.x + 256 * t;
-            const int mm = idx & (kPK - 1), uu = idx >> 4;  // a: 16 consecutive modes of one row
-            const int u = u0 + uu, m = m0 + mm;
-            As[mm][uu] = (u < U && m < M) ? a[(size_t)u * M + m] : 0.f;
-            const int ii = idx & (kPT - 1), mb = idx >> 7;  // basis: 128 consecutive pixels of one mode
-            const int i = i0 + ii, mbm = m0 + mb;
-            Bs[mb][ii] = (i < npix && mbm < M) ? basis[(size_t)mbm * npix + i] : 0.f;
+            for (int t = 0; t < kPT * kPK / 256; ++t) {
+                const int uu = au + 256 / kPK * t, mb = bm + 256 / kPT * t;
+                const bool la = u0 + uu < U && m0 + am < M, lb = i0 + bi < npix && m0 + mb < M;
+                copy_async4(&As[buf][am][uu], la ? a + (size_t)(u0 + uu) * M + m0 + am : a, la);
+                copy_async4(&Bs[buf][mb][bi], lb ? basis + (size_t)(m0 + mb) * npix + i0 + bi : basis, lb);
+            }
         }
-        __syncthreads();
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float2 eq[4][4], cr[4][4];  // rows 2 r, 2 r + 1 and pixels 2 c, 2 c + 1: (00, 11) and (01, 10)
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) eq[r][c] = cr[r][c] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int st = 0; st < kPStages - 1; ++st) fetch(st);
+    for (int step = 0; step < steps; ++step) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kPStages - 2) : "memory");
+        __syncthreads();  // this step's operands; and every thread is done with the step before
+        fetch(step + kPStages - 1);
+        const int buf = step % kPStages;
 #pragma unroll
         for (int k = 0; k < kPK; ++k) {
-            const float4 a0 = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
-            const float4 a1 = *reinterpret_cast<const float4*>(&As[k][64 + ty * 4]);
-            const float4 b0 = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
-            const float4 b1 = *reinterpret_cast<const float4*>(&Bs[k][64 + tx * 4]);
-            const float ar[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const float br[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+            float2 ar[4], br[4];
 #pragma unroll
-            for (int r = 0; r < 8; ++r)
+            for (int h = 0; h < 2; ++h) {
+                const float4 v = *reinterpret_cast<const float4*>(&As[buf][k][64 * h + ty * 4]);
+                const float4 w = *reinterpret_cast<const float4*>(&Bs[buf][k][64 * h + tx * 4]);
+                ar[2 * h] = make_float2(v.x, v.y);
+                ar[2 * h + 1] = make_float2(v.z, v.w);
+                br[2 * h] = make_float2(w.x, w.y);
+                br[2 * h + 1] = make_float2(w.z, w.w);
+            }
 #pragma unroll
-                for (int c = 0; c < 8; ++c) acc[r][c] = fmaf(ar[r], br[c], acc[r][c]);
+            for (int c = 0; c < 4; ++c) {
+                const float2 bs = make_float2(br[c].y, br[c].x);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    eq[r][c] = __ffma2_rn(ar[r], br[c], eq[r][c]);
+                    cr[r][c] = __ffma2_rn(ar[r], bs, cr[r][c]);
+                }
+            }
         }
-        __syncthreads();
     }
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
         const int u = u0 + (r < 4 ? ty * 4 + r : 64 + ty * 4 + r - 4);
         if (u >= U) continue;
         float* row = out + (size_t)u * npix;
+        float v[8];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const float2 e = eq[r / 2][c], x = cr[r / 2][c];
+            v[2 * c] = scale * (r & 1 ? x.y : e.x);
+            v[2 * c + 1] = scale * (r & 1 ? e.y : x.x);
+        }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int i = i0 + h * 64 + tx * 4;
             if (vec_store) {  // npix % 4 == 0 and a 16-byte aligned output: whole float4 in or out
                 if (i < npix)
-                    *reinterpret_cast<float4*>(row + i) =
-                        make_float4(scale * acc[r][4 * h], scale * acc[r][4 * h + 1], scale * acc[r][4 * h + 2],
-                                    scale * acc[r][4 * h + 3]);
+                    *reinterpret_cast<float4*>(row + i) = make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
             } else {
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
-                    if (i + c < npix) row[i + c] = scale * acc[r][4 * h + c];
+                    if (i + c < npix) row[i + c] = v[4 * h + c];
             }
         }
     }

@@ -117,3 +117,26 @@ def test_spectra_beyond_one_wave(n, h, w, overlap, border, frames):
     ref = omfbd.half_spectrum(opatches.spectra_from_frames(data.astype(np.float64), n, overlap, border))
     err = np.abs(d - ref).max() / np.abs(ref).max()
     assert err <= 1e-5, err
+
+
+@pytest.mark.parametrize("n_modes,diams,n_frames,n_patches", [
+    (1, (31.0,), 1, 1), (8, (33.0, 20.0), 3, 5),   # one step of modes; odd boxes, one tile of units and pixels
+    (25, (36.0,), 11, 12), (33, (28.0, 24.0), 12, 11),  # remainders in modes, units (132) and pixels
+    (136, (32.0,), 4, 32),                          # a whole tile of units, modes beyond the tensor-core tiles
+])
+def test_simt_projection_edges(n_modes, diams, n_frames, n_patches):
+    """The SIMT phase projection at the edges of its tiles and of its copies ahead, through the OTFs it leads to
+    (within 2e-6 of the oracle's, as for the other OTFs)."""
+    import numpy as np
+    import torch
+
+    from oracle import mfbd as omfbd
+    case = cases.make_case(n_pix=64, diams=diams, wavelengths=(6563.0, 8542.0)[:len(diams)], n_frames=n_frames,
+                           n_modes=n_modes, basis="zernike", n_patches=n_patches, seed=20250700 + n_modes)
+    a32, _, _ = _inputs(case)
+    plan = _plan_for(case, projection="simt")
+    assert plan.info()["tc_projection"] == 0
+    h = plan.otf(torch.from_numpy(a32).cuda()).cpu().numpy()
+    for p in range(n_patches):
+        for k, inter in enumerate(omfbd.otf_patch(case["setup"], a32[p].astype(np.float64))):
+            assert np.abs(h[p, k] - omfbd.half_spectrum(inter["H"])).max() <= 2e-6, (p, k)
