@@ -71,9 +71,9 @@ NCU_DRAM_BYTES_PER_UNIT = {"forward_passes": (71857152 + 503112704) / 9600,
 # the adjoint, from one capture (--metrics dram__bytes_read.sum,
 # dram__bytes_write.sum) of the first 48 patches of the 3969-patch field
 # (6144 units, 409 MB of spectra: larger than L2)
-NCU_DRAM_BYTES_PER_UNIT_128 = {"forward_passes": (67911680 + 344916992) / 6144,
-                               "adjoint_passes": (481574144 + 66861568) / 6144,
-                               "reduction": (818419968 + 364834048) / 6144}
+NCU_DRAM_BYTES_PER_UNIT_128 = {"forward_passes": (100531968 + 179673600) / 6144,
+                               "adjoint_passes": (494291456 + 85071872) / 6144,
+                               "reduction": (692017920 + 217249280) / 6144}
 # DRAM bytes per launch of the front-end kernels on the 961-patch 64 px field
 # (one ncu capture of the full launch each): spectra_tma_kernel (MemoryWorkload
 # section: 3.734345 TB/s x 121.088 us); object_image_kernel + merge_kernel
@@ -84,10 +84,10 @@ NCU_FRONT_DRAM_BYTES = {"spectra_from_frames": int(3.734345e12 * 121.088e-6),
                         "ls_filter_objects": 779402496 + 16724480 + 48732416 + 3328}
 # DRAM bytes of the batch kernel per 64 px-equivalent unit, from one ncu
 # capture of the first 200 problems of the 2000-problem batch (13869 units)
-# under the schedule the autotuner picks there (one launch, window 0, the
-# 170-register variant)
-NCU_BATCH_DRAM_BYTES_PER_UNIT64 = (1142750976 + 911612160) / 13868.964937802688
-NCU_BATCH_SCHEDULE = (0, 0, 1)  # mode, window_units, variant of that capture
+# under the schedule the autotuner picks on all of them (staged, five
+# launches, the 128-register variant)
+NCU_BATCH_DRAM_BYTES_PER_UNIT64 = (1102719232 + 633383936) / 13868.964937802688
+NCU_BATCH_SCHEDULE = (1, 0, 0)  # mode, window_units, variant of that capture
 METRIC = "loss+grad evals/s (patch*obj*frame units at 64px)"
 UNIT = "units/s"
 
@@ -277,11 +277,18 @@ def reduction_flops_per_unit(n_pix):
     return 36.0 * n_pix * (n_pix // 2 + 1)
 
 
-def reduction_bytes_per_unit(n_pix, n_frames, spec_cols):
+def reduction_bytes_per_unit(n_pix, n_frames, spec_cols, support=None):
     """Algorithmic bytes per unit of the frame reduction: D read, H read,
-    G written (complex64 half spectra), object written once per J frames."""
+    G written (complex64 half spectra; only `support` frequencies of them
+    where the kernel leaves the rest out), object written once per J frames."""
     half = n_pix * (n_pix // 2 + 1) * 8
-    return n_pix * spec_cols * 8 + 2 * half + half / n_frames
+    return n_pix * spec_cols * 8 + 2 * (half if support is None else 8 * support) + half / n_frames
+
+
+def half_spectrum_support(n_pix, diam):
+    """Half-spectrum frequencies within a pupil diameter of 0, the OTF's support."""
+    return sum(1 for y in range(-(n_pix // 2), n_pix // 2) for x in range(n_pix // 2 + 1)
+               if x * x + y * y < diam * diam)
 
 
 def measured_peaks():
@@ -785,7 +792,9 @@ def finish_line(args, plan, info, w, world, ms, value, e2e, prof, clk, peaks):
     units_obj = w["n_patches"] * w["n_frames"]
     fwd_flops = sum(f for f, _ in per_obj) * units_obj
     adj_flops = sum(a for _, a in per_obj) * units_obj
-    red_bytes = reduction_bytes_per_unit(w["n_pix"], w["n_frames"], w["n_pix"] // 2 + 1) * units_of(w)
+    # the general-size kernels touch H and G on the OTF's support only
+    support = None if w["n_pix"] == 64 else sum(half_spectrum_support(w["n_pix"], d) for d in w["diams"]) / len(w["diams"])
+    red_bytes = reduction_bytes_per_unit(w["n_pix"], w["n_frames"], w["n_pix"] // 2 + 1, support) * units_of(w)
     mp = measured_peaks()
     n_sm = torch.cuda.get_device_properties(local_rank).multi_processor_count
     alu_peak, alu_basis, alu_derived = alu_peak_of(peaks, n_sm)

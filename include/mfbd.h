@@ -80,17 +80,17 @@ typedef enum {
                                         * (comparison runs; not with MFBD_PREC_BF16_PHASE) */
 #define MFBD_FLAG_RECOMPUTE_BACKWARD 0x4u /* the adjoint recomputes the field F P instead of
                                            * keeping it from the forward pass: 8 N^2 fewer
-                                           * bytes of device memory per (patch, object, frame)
-                                           * (at N = 64 also the 8 W^2 of the pupil phasors),
+                                           * bytes of device memory per (patch, object, frame),
                                            * about a quarter more adjoint work */
 #define MFBD_FLAG_GENERIC_KERNELS 0x8u /* run N = 64 on the kernels of the other patch
-                                        * sizes (one CTA per unit) instead of the 64-pixel
-                                        * pass machine (comparison runs) */
+                                        * sizes (one CTA per unit) also where the fused
+                                        * kernel of that size applies (comparison runs) */
 #define MFBD_FLAG_SPLIT_PASSES 0x10u /* N = 64: run mfbd_loss_grad (and the explicit and
                                       * host-buffer calls) as three kernels that exchange
                                       * the OTFs, seeds, fields and phasors through the
                                       * plan's workspaces, instead of the fused kernel
-                                      * that keeps them on chip (comparison runs) */
+                                      * that keeps them on chip, or the general-size
+                                      * kernels (comparison runs) */
 
 typedef struct {
     int n_pix;      /* N, patch size in pixels: 48, 64, 96 or 128 */
@@ -116,14 +116,20 @@ typedef struct {
     int pupil_pixels[8];   /* n_pup,k: pixels inside pupil k */
     int pupil_box[8];      /* W_k: side of the pupil's bounding box */
     size_t workspace_bytes; /* device memory owned by the plan */
-    int slots_per_cta;      /* frames a CTA of the fused kernel works on at once */
-    int ctas;               /* CTAs of the fused kernel */
-    int reduction_split;    /* warps per (patch, object) of the frame reduction; > 1 adds a
-                               second launch that sums the per-split losses in order */
+    int slots_per_cta;      /* units (frames) a CTA of the 64 px pass machine works on at
+                               once; 0: the plan runs the general-size kernels */
+    int ctas;               /* its CTAs */
+    int reduction_split;    /* parts that the frame reduction cuts a (patch, object) into
+                               (warps on the 64 px pass machine, CTAs of 256 threads on the
+                               general-size kernels, whose losses a second launch adds in
+                               order) */
     int fused_ctas;         /* CTAs of the fused per-(patch, object) kernel that
-                               mfbd_loss_grad runs (one per SM), or 0 when it runs the
-                               three-kernel path (N != 64, J > 12, a pupil box wider
-                               than 37 px, or MFBD_FLAG_SPLIT_PASSES) */
+                               mfbd_loss_grad runs (one per SM; with too few pairs for
+                               that, a cluster of CTAs takes each), or 0 when it runs the
+                               passes and the reduction as kernels of their own (N != 64,
+                               J > 12, a pupil box wider than 37 px,
+                               MFBD_FLAG_SPLIT_PASSES, MFBD_FLAG_GENERIC_KERNELS or
+                               MFBD_FLAG_RECOMPUTE_BACKWARD) */
     int tc_projection;      /* 1: the phase projection phi = c B a runs on the tensor cores */
     int tc_adjoint;         /* 1: the modal adjoint dL/da = c B^T dL/dphi runs on the tensor
                                cores (dL/dphi and the basis split into three BF16 planes,
@@ -172,10 +178,13 @@ int mfbd_backward(mfbd_plan_t plan, float* grad, void* stream);
  * above. For N = 64 with J <= 12 and pupil boxes up to 37 px the pass work is
  * one fused launch (the fused per-(patch, object) kernel: forward passes,
  * frame reduction and adjoint passes of a pair in one CTA, the OTFs and seeds
- * in shared memory, the fields in a per-CTA buffer that stays in L2) plus a
- * small loss-combine kernel, between the modal phase projection and the
- * modal adjoint; otherwise the three-kernel path. Keeps nothing for
- * mfbd_backward on the fused path. */
+ * in shared memory, the fields in a per-CTA buffer that stays in L2; where
+ * the pairs are too few to fill the GPU, a cluster of CTAs takes each, with
+ * the same results bit for bit), between the modal phase projection and the
+ * modal adjoint; otherwise the forward passes, the frame reduction and the
+ * adjoint passes are launches of their own. Keeps nothing for mfbd_backward
+ * on the fused path. Outside stream capture the launches of a call may be
+ * chained (each kernel's set-up overlaps the end of the one before it). */
 int mfbd_loss_grad(mfbd_plan_t plan, const float* coeffs, const void* spectra,
                    double* loss, void* object, float* grad, void* stream);
 
@@ -413,7 +422,9 @@ typedef struct mfbd_batch* mfbd_batch_t;
 
 typedef struct {
     int n_problems;
-    long long n_patches, n_units, n_items;
+    long long n_patches, n_units;
+    long long n_items;       /* work items of the launch list (a patch's phases, reduction and
+                              * modal adjoint are cut into parts) */
     long long coeff_floats, spectra_complex, loss_doubles, object_complex;  /* packed sizes */
     size_t workspace_bytes;  /* device memory owned by the batch */
     int mode;                /* MFBD_BATCH_ONE_LAUNCH or MFBD_BATCH_STAGED */
@@ -449,8 +460,8 @@ int mfbd_batch_get_offsets(mfbd_batch_t batch, long long* coeffs, long long* spe
  * window_units (one launch: the kinds of item of about this many 64 px units
  * are interleaved with the next window's; <= 0: all items of a kind before
  * the next kind), ctas_per_sm (1..max_ctas_per_sm of the variant, 0: the
- * maximum), variant (0: the kernel compiled with up to 255 registers a
- * thread, 2 CTAs of 128 threads per SM; 1: up to 170 registers, 3 CTAs per
+ * maximum), variant (0: the kernel compiled with up to 128 registers a
+ * thread, 2 CTAs of 256 threads per SM; 1: up to 80 registers, 3 CTAs per
  * SM, the 96 and 128 px passes spilling). Synchronises the device (the work
  * list is rewritten). */
 int mfbd_batch_set_schedule(mfbd_batch_t batch, int mode, int window_units, int ctas_per_sm, int variant);

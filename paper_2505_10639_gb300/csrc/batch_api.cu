@@ -1,6 +1,6 @@
 // C ABI of uneven batches (mfbd_batch_*): validation, shared plan-time data,
 // packed layouts, the item list of a schedule, launches and the autotuner.
-// The arithmetic is in batch_kernels.cu and unit_passes.cuh.
+// The arithmetic is in batch_kernels.cuh, lane_passes.cuh and frame_reduction.cuh.
 #include "../../include/mfbd_testing.h"
 #include "batch_internal.h"
 #include "optics_host.h"

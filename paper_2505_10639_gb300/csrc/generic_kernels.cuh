@@ -1,5 +1,6 @@
 // Pass kernels of one problem for patch sizes other than 64 (48, 96, 128),
-// and for 64 on request: one CTA per unit (patch, object, frame),
+// and for 64 px plans outside the fused kernel's range (more than 12 frames,
+// pupil boxes over 37 px, recompute, on request): one CTA per unit (patch, object, frame),
 // persistent over the units. The passes themselves (Sec. 3.1, Eqs. 20-22 and
 // their adjoint) are in lane_passes.cuh. Each patch size is instantiated in a
 // translation unit of its own (generic_n48.cu ... generic_n128.cu) so that
