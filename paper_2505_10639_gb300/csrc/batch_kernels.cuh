@@ -235,7 +235,16 @@ __device__ void item_grad(const BatchParams& prm, const BatchProblem& pr, int p,
 
 // R part: the CTA's threads share the part's frequencies of each object; the
 // patch loss adds an object's warps in order, then the objects, then (the last
-// part to arrive) the parts.
+// part to arrive) the parts. The lanes that a frequency's frames are split over
+// follow from J alone, so that every kernel variant sums in the same order (and
+// the autotuner's choice cannot change the bits); HOLD, what the variant's
+// register budget holds, only decides whether a lane keeps its frames (16) or
+// reads them twice in chunks. (Splitting 9 to 16 frames over two lanes in the
+// 80-register variant alone read them once, with other bits: 400 problems of 48
+// and 64 px, for which that variant was the fastest, 812 us; now the other one
+// is, 859 us.)
+constexpr int kRedFrames = 16;  // frames of a frequency in a lane
+
 template <int HOLD>
 __device__ void item_reduce(const BatchParams& prm, const BatchProblem& pr, int p, int part, double* warps) {
     const int N = pr.N, NH = N / 2 + 1, J = pr.J, parts = red_parts(N);
@@ -260,9 +269,11 @@ __device__ void item_reduce(const BatchParams& prm, const BatchProblem& pr, int 
                                                           kF * (kBT / 32) * parts);
         };
         using fftreg::IC;
-        const double v = J <= HOLD       ? share(IC<1>{}, IC<HOLD>{})
-                         : J <= 2 * HOLD ? share(IC<2>{}, IC<HOLD>{})
-                                         : share(IC<1>{}, IC<0>{});
+        constexpr int kFull = HOLD >= kRedFrames ? HOLD : 0;
+        const double v = J <= HOLD             ? share(IC<1>{}, IC<HOLD>{})
+                         : J <= kRedFrames     ? share(IC<1>{}, IC<kFull>{})
+                         : J <= 2 * kRedFrames ? share(IC<2>{}, IC<kFull>{})
+                                               : share(IC<1>{}, IC<0>{});
         tot += cta_sum<kBT / 32>(v, warps);
         __syncthreads();
     }

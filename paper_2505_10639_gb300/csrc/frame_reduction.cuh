@@ -49,13 +49,13 @@ struct RedPtr {
 // HBM is the floor (D once, H and G once on the support); what it needs is
 // loads in flight and no second read: a frequency's frames are loaded once, all
 // at once, into the registers of its lanes (J <= HOLD FS), or (HOLD = 0, any J)
-// in chunks of kChunk frames, twice. Lanes outside the support take the same
+// in chunks of kChunk frames, twice; both add a lane's frames in order, so FS
+// alone decides the bits. Lanes outside the support take the same
 // way with their loads of H predicated off: a path of their own, which most
 // warps would run as well as the other, was slower (96 px 0.081 -> 0.100 ms).
 // The object-inferring loss (r.oin) needs FS = 1.
 template <int HOLD, int FS>
 __device__ __forceinline__ double reduce_lane(const RedPtr& r, int f0, int fstep) {
-    static_assert(FS == 1 || HOLD > 0, "frames are split over lanes in the register form only");
     constexpr int kChunk = 8, kF = 32 / FS;
     const int N = r.N, NH = N / 2 + 1, half = N * NH, J = r.J;
     const unsigned dstride = (unsigned)N * r.spec_ld;  // J * dstride < 2^32
@@ -132,26 +132,27 @@ __device__ __forceinline__ double reduce_lane(const RedPtr& r, int f0, int fstep
             } else {
                 auto chunks = [&](bool on, auto&& use) {
 #pragma unroll 1
-                    for (int j0 = 0; j0 < J; j0 += kChunk) {
+                    for (int j0 = 0; j0 < nj; j0 += kChunk) {
                         float2 d[kChunk], h[kChunk];
                         float wv[kChunk];
 #pragma unroll
                         for (int c = 0; c < kChunk; ++c) {
-                            const bool in = on && j0 + c < J;
+                            const bool in = on && j0 + c < nj;
                             d[c] = in ? dp[(unsigned)(j0 + c) * dstride] : make_float2(0.f, 0.f);
                             h[c] = in && sup ? hp[(unsigned)(j0 + c) * (unsigned)half] : make_float2(0.f, 0.f);
                             wv[c] = in ? wp[j0 + c] : 0.f;
                         }
 #pragma unroll
                         for (int c = 0; c < kChunk; ++c)
-                            if (j0 + c < J) use(d[c], h[c], wv[c], j0 + c);
+                            if (j0 + c < nj) use(d[c], h[c], wv[c], j0 + c);
                     }
                 };
                 chunks(true, [&](float2 d, float2 h, float wj, int) { gather(d, h, wj); });
+                const float own = e;  // this lane's share
                 fine = solve();
                 if (fine) {  // outside the support the residual is the data
                     chunks(sup, scatter);
-                    if (!sup) t = e;
+                    if (!sup) t = own;
                 }
             }
             if (!fine) {
