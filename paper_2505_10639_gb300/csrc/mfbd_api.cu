@@ -576,7 +576,7 @@ int run_fused(mfbd_plan_t p, int stages, const void* spectra, double* loss, void
 int run_pairs(mfbd_plan_t p, const void* spectra, double* loss, void* object, cudaStream_t s, int p0, int np) {
     FusedParams f = fused_params(p, p0, np, spectra, loss, object, nullptr, nullptr, nullptr);
     f.fscr = p->d_fscr;
-    f.lpair = p->d_lpair + (size_t)p0 * p->K * std::max(1, p->spread);
+    f.lpair = p->d_lpair + (size_t)p0 * p->K;
     f.csize = p->spread;
     f.lcnt = p->d_lcnt + p0;
     f.fticket = p->d_fticket;
@@ -911,8 +911,7 @@ int mfbd_plan_create(mfbd_plan_t* out, const mfbd_plan_desc* d, void* stream) {
                     p->fused_ctas = prop.multiProcessorCount * fper;
                     if ((st = dev_alloc(p, &p->d_fscr, (size_t)p->fused_ctas * kFusedFrames * n * n / 2))) throw st;
                     p->spread = spread_cluster(p->P, p->K, p->J, max_box);
-                    if ((st = dev_alloc(p, &p->d_lpair, (size_t)std::max(1, p->P * p->K) * std::max(1, p->spread))))
-                        throw st;
+                    if ((st = dev_alloc(p, &p->d_lpair, (size_t)std::max(1, p->P * p->K)))) throw st;
                     if ((st = dev_alloc(p, &p->d_lcnt, (size_t)std::max(1, p->P)))) throw st;
                     if ((st = dev_alloc(p, &p->d_fticket, 2))) throw st;
                     if ((e = cudaMemsetAsync(p->d_lcnt, 0, (size_t)std::max(1, p->P) * sizeof(int), s)) ||

@@ -89,8 +89,8 @@ int fused_pair_ctas_per_sm(int es);
 cudaError_t launch_fused_pairs(const FusedParams& prm, int es, int ctas, cudaStream_t s);
 
 // The same with a cluster of prm.csize CTAs per pair, for few pairs
-// (spread_kernels.cu); gscr holds the plan's per-unit OTF / seed buffers, lpair
-// P x K x csize losses. spread_cluster: the cluster size for a plan, 0 where the
+// (spread_kernels.cu), loss, object and dL/da the same bits; gscr holds the
+// plan's per-unit OTF / seed buffers. spread_cluster: the cluster size for a plan, 0 where the
 // fused kernel is the better one or the clusters do not fit.
 int spread_cluster(int P, int K, int J, int max_box);
 cudaError_t launch_spread_pairs(const FusedParams& prm, cudaStream_t s);

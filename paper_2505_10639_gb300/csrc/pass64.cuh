@@ -142,10 +142,8 @@ __device__ __forceinline__ void st_hint(float4* a, float4 v, uint64_t pol) {
 // kCancel sum_j w|D_j|^2, estimated from E - |N|^2/Q) it cancels badly in
 // FP32 (for J = 1, r = D gamma / Q everywhere the OTF is large), so such a
 // frequency is redone with N, Q, O and r_j in FP64 -- except DC, whose seed
-// is zero and whose loss term is exact enough in FP32. Each thread sums its
-// loss terms with Kahan compensation and returns them in FP64 (the callers
-// combine the threads' sums in a fixed order). The thread takes the
-// frequencies fstart, fstart + fstep, ... < N (N/2 + 1); hbase points at the
+// is zero and whose loss term is exact enough in FP32. term(f, x) gets the
+// frequency's share x of the loss. The thread takes the frequencies fstart, fstart + fstep, ... < N (N/2 + 1); hbase points at the
 // pair's first frame of H (frames kHalf elements apart, global or shared
 // memory).
 // JM > 0: J <= JM, the J spectra and OTFs of a frequency are loaded once, all
@@ -153,9 +151,9 @@ __device__ __forceinline__ void st_hint(float4* a, float4 v, uint64_t pol) {
 // MODE: 0 takes the object-inferring branch when prm.oin is set, 1 compiles
 // the Wiener loss only, 2 the object-inferring loss only. STREAM: the
 // spectra are read with an L2 evict-first hint (JM > 0).
-template <int JM, int MODE = 0, bool STREAM = false>
-__device__ __forceinline__ double reduce_frequencies(const FusedParams& prm, int p, int k, float2* hbase,
-                                                     int fstart, int fstep) {
+template <int JM, int MODE, bool STREAM, class Term>
+__device__ __forceinline__ void each_frequency(const FusedParams& prm, int p, int k, float2* hbase, int fstart,
+                                               int fstep, Term&& term) {
     const int J = prm.J;
     const size_t unit0 = ((size_t)p * prm.K + k) * J;
     const size_t dstride = (size_t)kN * prm.spec_ld;
@@ -169,7 +167,6 @@ __device__ __forceinline__ double reduce_frequencies(const FusedParams& prm, int
         for (int j = 0; j < JM; ++j) wv[j] = (j < J) ? w[j] : 0.f;
     }
     const uint64_t pol = STREAM ? l2_evict_first() : 0;
-    KahanSum acc;
     for (int f = fstart; f < kHalf; f += fstep) {
         const int ky = f / kNH, kx = f - ky * kNH;
         const size_t doff = (size_t)ky * prm.spec_ld + kx;
@@ -194,7 +191,7 @@ __device__ __forceinline__ double reduce_frequencies(const FusedParams& prm, int
             } else {
                 t = explicit_frequency(J, dp, dstride, hp, kHalf, w, prm.gamma, seed, prm.oin[ooff + doff], g);
             }
-            acc.add((kx == 0 || kx == kN / 2) ? t : 2.0f * t);
+            term(f, (kx == 0 || kx == kN / 2) ? t : 2.0f * t);
             if (prm.gobj) {
                 prm.gobj[ooff + doff] = g;
                 if (prm.spec_ld == kN && kx > 0 && kx < kN / 2)
@@ -269,7 +266,7 @@ __device__ __forceinline__ double reduce_frequencies(const FusedParams& prm, int
                 t = tsum + gam * (o.x * o.x + o.y * o.y);
             }
         }
-        acc.add((kx == 0 || kx == kN / 2) ? t : 2.0f * t);
+        term(f, (kx == 0 || kx == kN / 2) ? t : 2.0f * t);
         if (prm.object) {
             float2* ob = prm.object + ((size_t)p * prm.K + k) * dstride;
             ob[doff] = o;
@@ -277,6 +274,15 @@ __device__ __forceinline__ double reduce_frequencies(const FusedParams& prm, int
                 ob[(size_t)((kN - ky) % kN) * kN + (kN - kx)] = cconj(o);
         }
     }
+}
+
+// The same, the thread's loss terms summed with Kahan compensation and
+// returned in FP64 (the callers combine the threads' sums in a fixed order).
+template <int JM, int MODE = 0, bool STREAM = false>
+__device__ __forceinline__ double reduce_frequencies(const FusedParams& prm, int p, int k, float2* hbase, int fstart,
+                                                     int fstep) {
+    KahanSum acc;
+    each_frequency<JM, MODE, STREAM>(prm, p, k, hbase, fstart, fstep, [&](int, float x) { acc.add(x); });
     return (double)acc.s - (double)acc.c;
 }
 

@@ -13,9 +13,12 @@
 //
 // The transforms and every elementwise step are those of the fused kernel and
 // of the three-kernel path in the same order: object and dL/da agree with both
-// bit for bit. For that the twiddle products across lanes round as the compiler
-// contracts twmul's constant ones (fused_over_s; the pupil columns beyond
-// 32, which the other kernels transform by fft64_quarters, go through it here).
+// bit for bit. So does the loss with the fused kernel's: every CTA puts the
+// terms of its frequencies into the shared memory of the cluster's last one,
+// which adds them in the order of the fused kernel's threads. For that the
+// twiddle products across lanes round as the compiler contracts twmul's
+// constant ones (fused_over_s; the pupil columns beyond 32, which the other
+// kernels transform by fft64_quarters, go through it here).
 // Stating those roundings in twmul itself would tie the kernels together by
 // construction, but made the fused kernel 1 % slower.
 #include "chained.cuh"
@@ -206,10 +209,13 @@ __device__ __forceinline__ void frame_forward(const ObjParams& ob, const float* 
     __syncthreads();
 }
 
-// Adjoint passes of one frame: h (the seed G) -> gphi.
+// Adjoint passes of one frame: h (the seed G) -> gphi. The first two occupy the
+// lower warps; the upper four (128 threads) run beside(0) and, a CTA barrier
+// later, beside(1).
+template <class Beside>
 __device__ __forceinline__ void frame_adjoint(const ObjParams& ob, const float* __restrict__ ph,
                                               float* __restrict__ gphi, float2* E, const float2* field,
-                                              const float2* h) {
+                                              const float2* h, Beside&& beside) {
     const Lane t;
     float* Ef = reinterpret_cast<float*>(E);
     const int W = ob.W;
@@ -226,6 +232,8 @@ __device__ __forceinline__ void frame_adjoint(const ObjParams& ob, const float* 
         fft64_lanes(a, t.l);
 #pragma unroll
         for (int k = 0; k < kQ; ++k) E[row_base(16 * t.q) + k * kLd + kx + (kx >> 4)] = a[k];
+    } else {
+        beside(0);
     }
     __syncthreads();
     if (t.line < kN / 2) {  // C2R: conj of T_i + i T_(i+32), Hermitian-extended; g_q rows as floats
@@ -252,6 +260,8 @@ __device__ __forceinline__ void frame_adjoint(const ObjParams& ob, const float* 
             g0[k] = a[k].x * sc;
             g1[k] = a[k].y * -sc;
         }
+    } else {
+        beside(1);
     }
     __syncthreads();
     {  // rows of conj(g_q p), transformed; the box columns kept
@@ -305,15 +315,29 @@ __device__ __forceinline__ void cluster_sync() {
 constexpr int kSpreadFrames = 2;  // frames of a CTA
 constexpr size_t kSpreadSmem = (kBufElems + (size_t)kSpreadFrames * kQ * kST) * sizeof(float2);
 
+// Address of this CTA's shared-memory object in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t in_rank(const void* p, int rank) {
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return a;
+}
+
 // EXPL: the object-inferring loss. Cluster c of prm.csize CTAs carries pair c.
 template <bool EXPL>
 __global__ void __launch_bounds__(kST, 2) spread_pair_kernel(const FusedParams prm) {
     extern __shared__ __align__(16) unsigned char spsm[];
-    __shared__ double swarp[kSW];
+    // The last CTA sums the pair's loss: chain c adds the terms c, c + kChains,
+    // ... as thread c of the fused kernel does, so a patch's loss does not depend
+    // on which of the two kernels its plan takes. Half its warps do so beside the
+    // first adjoint passes (1 pair of 8 frames: 43.6 us an evaluation; the sum before
+    // them 45.7, each CTA summing its own frequencies, with other bits, 44.5).
+    constexpr int kChains = 32 * kFusedFrames;
+    __shared__ float terms[kHalf];
+    __shared__ double swarp[kFusedFrames];
     float2* E = reinterpret_cast<float2*>(spsm);
     float2* field = E + kBufElems;
     const int csize = prm.csize;
-    const int rank = (int)(blockIdx.x % csize), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = (int)(blockIdx.x % csize), lane = threadIdx.x & 31;
     const long long pair = blockIdx.x / csize;
     const int J = prm.J, K = prm.K;
     const long long p = pair / K;
@@ -329,38 +353,44 @@ __global__ void __launch_bounds__(kST, 2) spread_pair_kernel(const FusedParams p
                           field + (size_t)f * kQ * kST, hpair + (size_t)j * kHalf);
     }
     cluster_sync();  // every frame's OTF
-    double v = reduce_frequencies<kFusedFrames, EXPL ? 2 : 1, false>(prm, (int)p, k, hpair, rank * kST + threadIdx.x,
-                                                                     csize * kST);
+    const uint32_t sums = in_rank(terms, csize - 1);
+    each_frequency<kFusedFrames, EXPL ? 2 : 1, false>(
+        prm, (int)p, k, hpair, rank * kST + threadIdx.x, csize * kST,
+        [&](int f, float x) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(sums + 4 * f), "f"(x) : "memory"); });
+    cluster_sync();  // every seed and term of the loss
+    auto sum_loss = [&](int step) {  // the upper four warps of the last CTA
+        if (step == 0) {
+            for (int c = threadIdx.x - kST / 2; c < kChains; c += kST / 2) {  // whole warps
+                KahanSum acc;
+                for (int f = c; f < kHalf; f += kChains) acc.add(terms[f]);
+                double v = (double)acc.s - (double)acc.c;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if (lane == 0) swarp[warp] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int w = 0; w < kSW; ++w) tot += swarp[w];
-        prm.lpair[pair * csize + rank] = tot;
-    }
-    cluster_sync();  // every seed and share of the loss
-    if (rank == 0 && threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int r = 0; r < csize; ++r) tot += __ldcg(&prm.lpair[pair * csize + r]);
-        __stcg(&prm.lpair[pair * csize], tot);
-        // the pair that finishes the patch sums its objects in order and resets the count
-        __threadfence();
-        if (atomicAdd(&prm.lcnt[p], 1) == K - 1) {
+                for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+                if (lane == 0) swarp[c >> 5] = v;
+            }
+        } else if (threadIdx.x == kST / 2) {
+            double tot = 0.0;
+            for (int w = 0; w < kFusedFrames; ++w) tot += swarp[w];
+            __stcg(&prm.lpair[pair], tot);
+            // the pair that finishes the patch sums its objects in order and resets the count
             __threadfence();
-            double sum = 0.0;
-            for (int kk = 0; kk < K; ++kk) sum += __ldcg(&prm.lpair[(p * K + kk) * csize]);
-            prm.loss[p] = sum;
-            prm.lcnt[p] = 0;
+            if (atomicAdd(&prm.lcnt[p], 1) == K - 1) {
+                __threadfence();
+                double sum = 0.0;
+                for (int kk = 0; kk < K; ++kk) sum += __ldcg(&prm.lpair[p * K + kk]);
+                prm.loss[p] = sum;
+                prm.lcnt[p] = 0;
+            }
         }
-    }
+    };
     for (int f = 0; f < kSpreadFrames; ++f) {
         const int j = rank + f * csize;
         const long long img = ob.phi_off + (p * J + j) * ob.phi_unit + ob.phi_org;
         if (j < J)
             frame_adjoint(ob, prm.phi + img, prm.gphi + img, E, field + (size_t)f * kQ * kST,
-                          hpair + (size_t)j * kHalf);
+                          hpair + (size_t)j * kHalf, [&](int step) {
+                              if (f == 0 && rank == csize - 1) sum_loss(step);
+                          });
     }
 }
 
