@@ -70,6 +70,7 @@ struct mfbd_plan {
     bool fused = false;         // mfbd_loss_grad runs the fused per-(patch, object) kernel
     int fused_ctas = 0;         // its CTAs (one per SM)
     int spread = 0;             // few pairs: CTAs of the cluster that takes each instead (spread_kernels.cu)
+    bool spread_chain = false;  // and whether their launch may be chained
     float2* d_fscr = nullptr;   // its field slots [fused_ctas][kFusedFrames][N*N/2] (rows N/2..N-1)
     double* d_lpair = nullptr;  // its per-(patch, object) losses [P][K]
     int* d_lcnt = nullptr;      // its per-patch counts of finished objects [P], 0 between calls
@@ -584,7 +585,10 @@ int run_pairs(mfbd_plan_t p, const void* spectra, double* loss, void* object, cu
     for (int k = 0; k < p->K; ++k) f.korder[k] = k;
     std::stable_sort(f.korder, f.korder + p->K, [&](int a, int b) { return p->obj[a].W > p->obj[b].W; });
     const int pi = prof_begin(p, 5, s);
-    if (p->spread) f.gscr = p->d_gscr;
+    if (p->spread) {
+        f.gscr = p->d_gscr;
+        f.chain = p->chain && p->spread_chain;
+    }
     const cudaError_t e =
         p->spread ? launch_spread_pairs(f, s) : launch_fused_pairs(f, p->geo.xs, p->fused_ctas, s);
     prof_end(p, pi, s, 1);
@@ -910,7 +914,7 @@ int mfbd_plan_create(mfbd_plan_t* out, const mfbd_plan_desc* d, void* stream) {
                     p->fused = true;
                     p->fused_ctas = prop.multiProcessorCount * fper;
                     if ((st = dev_alloc(p, &p->d_fscr, (size_t)p->fused_ctas * kFusedFrames * n * n / 2))) throw st;
-                    p->spread = spread_cluster(p->P, p->K, p->J, max_box);
+                    p->spread = spread_cluster(p->P, p->K, p->J, max_box, &p->spread_chain);
                     if ((st = dev_alloc(p, &p->d_lpair, (size_t)std::max(1, p->P * p->K)))) throw st;
                     if ((st = dev_alloc(p, &p->d_lcnt, (size_t)std::max(1, p->P)))) throw st;
                     if ((st = dev_alloc(p, &p->d_fticket, 2))) throw st;

@@ -90,9 +90,10 @@ cudaError_t launch_fused_pairs(const FusedParams& prm, int es, int ctas, cudaStr
 
 // The same with a cluster of prm.csize CTAs per pair, for few pairs
 // (spread_kernels.cu), loss, object and dL/da the same bits; gscr holds the
-// plan's per-unit OTF / seed buffers. spread_cluster: the cluster size for a plan, 0 where the
-// fused kernel is the better one or the clusters do not fit.
-int spread_cluster(int P, int K, int J, int max_box);
+// plan's per-unit OTF / seed buffers. spread_cluster: the cluster size for a
+// plan, 0 where the fused kernel is the better one or the clusters do not fit;
+// *chain: whether its launch may be chained.
+int spread_cluster(int P, int K, int J, int max_box, bool* chain);
 cudaError_t launch_spread_pairs(const FusedParams& prm, cudaStream_t s);
 
 // phase[u][i] += div[u mod J][i] for U units (U a multiple of J): the

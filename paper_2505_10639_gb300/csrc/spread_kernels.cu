@@ -425,11 +425,24 @@ cudaError_t launch_spread(const FusedParams& prm, cudaStream_t s, int* clusters)
 
 // One frame per CTA if all pairs are then resident at once, else (more than 8
 // frames, where the fused kernel runs three warps a scheduler) two; beyond that
-// the fused kernel. us per evaluation, this kernel and the fused one: 1 pair of
-// 8 frames 44 and 66, 32 of 6 frames 51 and 64, 16 of 12 frames 51 and 92; two
-// frames to a CTA: 40 pairs of 12 frames 71 and 88, but 64 of 6 frames 72 and 64.
-// A second wave is slower (48 pairs of 12 frames 115 and 88).
-int spread_cluster(int P, int K, int J, int max_box) {
+// the fused kernel. us per evaluation, this kernel and the fused one, both with
+// chained launches: 1 pair of 8 frames 44 and 69, 41 of 6 frames 57 and 83, 20 of
+// 12 frames 50 and 91; two frames to a CTA: 40 pairs of 12 frames 73 and 87, but
+// 64 of 6 frames 72 and 64. A second wave is slower (48 pairs of 12 frames 115
+// and 88).
+//
+// chain: whether the kernel may be launched over the projection's tail. Its
+// clusters then go to the SMs that are already free. While they are few, that
+// saves 2 to 3 us (15 pairs of 12 frames 50 against 52); near the most that fit,
+// what the projection's CTAs leave is cut up and a second wave forms: 28 pairs of
+// 10 frames 74 us chained, 52 not, 83 on the fused kernel; 45 pairs of 12 frames
+// (28 px) 108, 71, 75. A second wave was seen from 80 % of the clusters that fit
+// up, so the line is at three quarters; clusters of two take the two places of
+// an SM and always fit (152 pairs 65 and 68 us). Single CTAs (one frame) double
+// up on the free SMs as soon as they are nearly as many as all SMs: 130 pairs 85
+// and 87 us, 142 pairs 112 and 87, the fused kernel 101; there the line is at 0.8
+// of the SMs.
+int spread_cluster(int P, int K, int J, int max_box, bool* chain) {
     if (J > kFusedFrames || max_box > kMaxBox || P < 1 || (long long)P * K > 4096) return 0;
     for (int frames = 1; frames <= (J > 8 ? kSpreadFrames : 1); ++frames) {
         FusedParams prm{};
@@ -440,7 +453,11 @@ int spread_cluster(int P, int K, int J, int max_box) {
         const bool ok = launch_spread<false>(prm, nullptr, &n0) == cudaSuccess &&
                         launch_spread<true>(prm, nullptr, &n1) == cudaSuccess;
         if (!ok) cudaGetLastError();
-        if (ok && (long long)P * K <= std::min(n0, n1)) return prm.csize;
+        const long long pairs = (long long)P * K, fit = std::min(n0, n1);
+        if (ok && pairs <= fit) {
+            *chain = prm.csize == 2 || (4 * pairs <= 3 * fit && (prm.csize > 1 || 5 * pairs <= 2 * fit));
+            return prm.csize;
+        }
     }
     return 0;
 }

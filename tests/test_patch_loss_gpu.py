@@ -36,3 +36,25 @@ def test_patch_loss_and_object_by_plan_size(frames, diams, full):
     few.check()
     many.check()
     assert np.isfinite(lf.cpu().numpy()).all()
+
+
+@pytest.mark.parametrize("frames,diam,sizes", [
+    (1, 36.0, (60, 142, 200)), (4, 28.0, (30, 70)), (10, 36.0, (11, 28)), (12, 28.0, (9, 22, 45)),
+])
+def test_patch_results_across_the_cluster_rule(frames, diam, sizes):
+    """Plan sizes well below and near the most clusters that fit the GPU at once (where the launch is not chained, or
+    a CTA takes two frames): the bits of a single patch's plan, call after call."""
+    case = cases.make_case(diams=(diam,), wavelengths=(6563.0,), n_frames=frames, n_modes=9, basis="zernike",
+                           n_patches=1, seed=20251300 + frames)
+    a32, d32, _ = _inputs(case)
+    a, d = torch.from_numpy(a32).cuda(), torch.from_numpy(d32).cuda()
+    one = _plan_for(case, n_patches=1)
+    l1, _, o1 = one.loss_grad(a, d, want_object=True)
+    for n in sizes:
+        plan = _plan_for(case, n_patches=n)
+        an, dn = a.repeat(n, 1, 1), d.repeat(n, 1, 1, 1, 1)
+        out = [plan.loss_grad(an, dn, want_object=True) for _ in range(6)]
+        plan.check()
+        for ln, gn, on in out:
+            assert torch.equal(ln, l1.repeat(n)) and torch.equal(on, o1.repeat(n, 1, 1, 1)), n
+            assert torch.equal(gn, gn[:1].repeat(n, 1, 1)), n
