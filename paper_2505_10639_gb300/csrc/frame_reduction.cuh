@@ -53,9 +53,10 @@ struct RedPtr {
 // alone decides the bits. Lanes outside the support take the same
 // way with their loads of H predicated off: a path of their own, which most
 // warps would run as well as the other, was slower (96 px 0.081 -> 0.100 ms).
-// The object-inferring loss (r.oin) needs FS = 1.
-template <int HOLD, int FS>
+// EXPL: the object-inferring loss (r.oin), FS = 1.
+template <int HOLD, int FS, bool EXPL = false>
 __device__ __forceinline__ double reduce_lane(const RedPtr& r, int f0, int fstep) {
+    static_assert(FS == 1 || !EXPL, "the object-inferring loss is not split over lanes");
     constexpr int kChunk = 8, kF = 32 / FS;
     const int N = r.N, NH = N / 2 + 1, half = N * NH, J = r.J;
     const unsigned dstride = (unsigned)N * r.spec_ld;  // J * dstride < 2^32
@@ -74,10 +75,24 @@ __device__ __forceinline__ double reduce_lane(const RedPtr& r, int f0, int fstep
         const float* wp = r.w + jb;
         const bool sup = wbit(r.supp, r.sw, ky, kx), seed = sup && f != 0;
         const float twice = (kx == 0 || kx == N / 2) ? 1.f : 2.f;
-        float2 o = FS == 1 && r.oin ? r.oin[doff] : make_float2(0.f, 0.f), g = make_float2(gam * o.x, gam * o.y);
+        float2 o = EXPL ? r.oin[doff] : make_float2(0.f, 0.f), g = make_float2(gam * o.x, gam * o.y);
         float t = 0.f;
-        if (FS == 1 && r.oin && sup) {  // object-inferring loss: the object is given
-            t = explicit_frequency(J, dp, dstride, hp, half, r.w, r.gamma, seed, o, g);
+        constexpr int kHeld = HOLD > 0 ? HOLD : 1;
+        float2 d[kHeld], h[kHeld];
+        float wv[kHeld];
+        if constexpr (HOLD > 0) {
+#pragma unroll
+            for (int j = 0; j < HOLD; ++j) {
+                const bool in = j < nj;
+                d[j] = in ? dp[(unsigned)j * dstride] : make_float2(0.f, 0.f);
+                h[j] = in && sup ? hp[(unsigned)j * (unsigned)half] : make_float2(0.f, 0.f);
+                wv[j] = in ? wp[j] : 0.f;
+            }
+        }
+        if (EXPL && sup) {  // the object is given
+            if constexpr (HOLD > 0)
+                t = explicit_held<HOLD>(J, d, h, wv, dp, dstride, hp, half, r.w, r.gamma, seed, o, g);
+            else t = explicit_frequency(J, dp, dstride, hp, half, r.w, r.gamma, seed, o, g);
         } else {
             float2 num = make_float2(0.f, 0.f);
             float e = 0.f, qs = 0.f;
@@ -95,31 +110,25 @@ __device__ __forceinline__ double reduce_lane(const RedPtr& r, int f0, int fstep
             };
             // false where the residual cancels (seed frequencies only)
             auto solve = [&]() {
-                if (FS == 1 && r.oin) return true;  // outside the support: the data's energy, O as given
+                if constexpr (EXPL) {
+                    return true;  // outside the support: the data's energy, O as given
+                } else {
 #pragma unroll
-                for (int off = kF; off < 32; off <<= 1) {
-                    num.x += __shfl_xor_sync(0xffffffffu, num.x, off);
-                    num.y += __shfl_xor_sync(0xffffffffu, num.y, off);
-                    e += __shfl_xor_sync(0xffffffffu, e, off);
-                    qs += __shfl_xor_sync(0xffffffffu, qs, off);
+                    for (int off = kF; off < 32; off <<= 1) {
+                        num.x += __shfl_xor_sync(0xffffffffu, num.x, off);
+                        num.y += __shfl_xor_sync(0xffffffffu, num.y, off);
+                        e += __shfl_xor_sync(0xffffffffu, e, off);
+                        qs += __shfl_xor_sync(0xffffffffu, qs, off);
+                    }
+                    qs += gam;
+                    const float invq = 1.0f / qs;
+                    o = cscale(num, invq);
+                    const float t_est = e - (num.x * num.x + num.y * num.y) * invq;
+                    return !(seed && t_est < kCancel * e);
                 }
-                qs += gam;
-                const float invq = 1.0f / qs;
-                o = cscale(num, invq);
-                const float t_est = e - (num.x * num.x + num.y * num.y) * invq;
-                return !(seed && t_est < kCancel * e);
             };
             bool fine;
             if constexpr (HOLD > 0) {
-                float2 d[HOLD], h[HOLD];
-                float wv[HOLD];
-#pragma unroll
-                for (int j = 0; j < HOLD; ++j) {
-                    const bool in = j < nj;
-                    d[j] = in ? dp[(unsigned)j * dstride] : make_float2(0.f, 0.f);
-                    h[j] = in && sup ? hp[(unsigned)j * (unsigned)half] : make_float2(0.f, 0.f);
-                    wv[j] = in ? wp[j] : 0.f;
-                }
 #pragma unroll
                 for (int j = 0; j < HOLD; ++j)
                     if (j < nj) gather(d[j], h[j], wv[j]);
@@ -169,7 +178,7 @@ __device__ __forceinline__ double reduce_lane(const RedPtr& r, int f0, int fstep
             r.obj[doff] = o;
             if (r.spec_ld == N && kx > 0 && kx < N / 2) r.obj[(size_t)((N - ky) % N) * N + (N - kx)] = cconj(o);
         }
-        if (FS == 1 && r.gobj) {
+        if (EXPL && r.gobj) {
             r.gobj[doff] = g;
             if (r.spec_ld == N && kx > 0 && kx < N / 2) r.gobj[(size_t)((N - ky) % N) * N + (N - kx)] = cconj(g);
         }

@@ -22,7 +22,7 @@ using namespace reduction;
 // px 0.852 -> 0.442 (60 % of the copy peak on what it cannot do without).
 constexpr int kRedWarps = 8;
 
-template <int HOLD, int FS>
+template <int HOLD, int FS, bool EXPL = false>
 __global__ void __launch_bounds__(32 * kRedWarps, HOLD == 32 ? 1 : 2) generic_reduce_kernel(const GenericParams prm) {
     constexpr int kF = 32 / FS;  // frequencies of a warp
     __shared__ double part[kRedWarps];
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(32 * kRedWarps, HOLD == 32 ? 1 : 2) generic_re
         r.oin = prm.oin ? prm.oin + (size_t)pk * dstride : nullptr;
         r.gobj = prm.gobj ? prm.gobj + (size_t)pk * dstride : nullptr;
         const double v = cta_sum<kRedWarps>(
-            reduce_lane<HOLD, FS>(r, kF * (kRedWarps * s + (threadIdx.x >> 5)), kF * kRedWarps * S), part);
+            reduce_lane<HOLD, FS, EXPL>(r, kF * (kRedWarps * s + (threadIdx.x >> 5)), kF * kRedWarps * S), part);
         if (threadIdx.x == 0) (prm.K * S == 1 ? prm.loss : prm.lpart)[u] = v;
         __syncthreads();
     }
@@ -115,10 +115,14 @@ cudaError_t launch_generic_reduction(const GenericParams& prm, int sms, cudaStre
     // lanes a frequency, then chunks: 2,904 units of 12 frames (96 px) 0.081 ms
     // (0.110 in chunks, 0.097 over two lanes of 8); 12,800 of 32 frames (128 px)
     // 0.442 (0.460 as 32 in one lane, 0.477 in chunks); 22,500 of 100 frames (64
-    // px) 0.283 (0.329 in chunks). The object-inferring form is not split.
-    auto kern = prm.J <= 8     ? generic_reduce_kernel<8, 1>
+    // px) 0.283 (0.329 in chunks). The object-inferring form is not split; held
+    // against read twice, whole evaluations: 900 patches of 15 frames (64 px) 824
+    // -> 707 us, 100 of 16 167 -> 154, 225 of 12 (96 px) 387 -> 345.
+    auto kern = prm.oin        ? (prm.J <= 8    ? generic_reduce_kernel<8, 1, true>
+                                  : prm.J <= 16 ? generic_reduce_kernel<16, 1, true>
+                                                : generic_reduce_kernel<0, 1, true>)
+                : prm.J <= 8   ? generic_reduce_kernel<8, 1>
                 : prm.J <= 16  ? generic_reduce_kernel<16, 1>
-                : prm.oin      ? generic_reduce_kernel<0, 1>
                 : prm.J <= 32  ? generic_reduce_kernel<16, 2>
                 : prm.J <= 64  ? generic_reduce_kernel<16, 4>
                 : prm.J <= 128 ? generic_reduce_kernel<32, 4>
