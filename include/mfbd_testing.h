@@ -23,6 +23,8 @@ extern "C" {
  *   6  complex adjoint, length 64, radix-4 network
  *   7  complex forward, length 48 (three 16-point FFTs and a radix-3 stage)
  *   8  complex adjoint, length 48
+ *   9  complex forward, length 6, a lane's share of a 48-point line
+ *  10  complex forward, length 12, a lane's share of a 96-point line
  * Forward: X[k] = sum x[n] exp(-2 pi i n k / N); adjoint uses exp(+...).
  * Returns 0 (MFBD_OK) or 1 (MFBD_ERR_INVALID_ARG) for an unknown kind or
  * NULL pointers. */

@@ -1,6 +1,22 @@
 // Host-side execution of the register FFTs (see include/mfbd_testing.h).
 #include "../../include/mfbd_testing.h"
 #include "fft_reg.cuh"
+#include "lane8.cuh"
+
+namespace {
+
+template <int R>
+void lane_dft(const float* in, float* out) {
+    float2 a[R];
+    for (int i = 0; i < R; ++i) a[i] = make_float2(in[2 * i], in[2 * i + 1]);
+    mfbd_dev::lane8::dft<R>(a);
+    for (int i = 0; i < R; ++i) {
+        out[2 * i] = a[i].x;
+        out[2 * i + 1] = a[i].y;
+    }
+}
+
+}  // namespace
 
 extern "C" int mfbd_test_fft_host(int kind, const float* in, float* out) {
     if (!in || !out) return 1;
@@ -55,6 +71,8 @@ extern "C" int mfbd_test_fft_host(int kind, const float* in, float* out) {
             for (int i = 0; i < 48; ++i) { out[2 * i] = a[i].x; out[2 * i + 1] = a[i].y; }
             return 0;
         }
+        case 9: lane_dft<6>(in, out); return 0;
+        case 10: lane_dft<12>(in, out); return 0;
         default:
             return 1;
     }
