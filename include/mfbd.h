@@ -180,7 +180,8 @@ int mfbd_backward(mfbd_plan_t plan, float* grad, void* stream);
  * frame reduction and adjoint passes of a pair in one CTA, the OTFs and seeds
  * in shared memory, the fields in a per-CTA buffer that stays in L2; where
  * the pairs are too few to fill the GPU, a cluster of CTAs takes each, with
- * the same results bit for bit), between the modal phase projection and the
+ * the same bits of loss and object: a patch's do not depend on how many
+ * patches its plan holds), between the modal phase projection and the
  * modal adjoint; otherwise the forward passes, the frame reduction and the
  * adjoint passes are launches of their own. Keeps nothing for mfbd_backward
  * on the fused path. Outside stream capture the launches of a call may be
@@ -462,8 +463,8 @@ int mfbd_batch_get_offsets(mfbd_batch_t batch, long long* coeffs, long long* spe
  * the next kind), ctas_per_sm (1..max_ctas_per_sm of the variant, 0: the
  * maximum), variant (0: the kernel compiled with up to 128 registers a
  * thread, 2 CTAs of 256 threads per SM; 1: up to 80 registers, 3 CTAs per
- * SM, the 96 and 128 px passes spilling). Synchronises the device (the work
- * list is rewritten). */
+ * SM, the 96 and 128 px passes spilling). Every schedule and variant gives the
+ * same bits. Synchronises the device (the work list is rewritten). */
 int mfbd_batch_set_schedule(mfbd_batch_t batch, int mode, int window_units, int ctas_per_sm, int variant);
 
 /* Loss, object (or NULL) and dL/da of every problem (layouts above),

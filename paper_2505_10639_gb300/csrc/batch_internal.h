@@ -48,7 +48,7 @@ struct BatchProblem {
 
 // Work items. F and A cover one unit (patch, object, frame), or several
 // consecutive units k J + j of one patch when N <= 64 (kSmallUnits);
-// P, R and G cover one patch.
+// P, R and G cover a part of one patch.
 enum BatchKind : int {
     BK_PROJ = 0,   // phases of every object and frame of a patch (Eq. 22)
     BK_FWD = 1,    // forward passes of a unit (Eqs. 20-21, OTF)

@@ -1,6 +1,6 @@
 // Batched persistent kernel: the whole loss + gradient of an uneven batch of
 // problems (patch sizes 48, 64, 96, 128; objects, frames and modes per
-// problem) in one launch.
+// problem) in one launch, or (staged) in one launch per kind of item.
 //
 // The work is a list of items, each of one kind (BatchKind), those of a whole
 // patch cut into parts: P, the phases
@@ -22,8 +22,9 @@
 // buffer and named barrier. Larger patches use all eight warps on one unit.
 // The passes are those of lane_passes.cuh. Measured on 500 drawn problems
 // (15,788 units): 6.76 ms with a unit per warp (N <= 64) or per 128 threads
-// and one or two lanes a line, 3.59 ms with these; F 1.17 -> 0.52, A 1.52 ->
-// 0.70 ms of the staged schedule.
+// and one or two lanes a line, 3.59 ms with these, 1.98 ms with P, R and G in
+// parts; staged P 0.87 -> 0.16, F 1.17 -> 0.51, R 2.04 -> 0.36, A 1.52 -> 0.68, G
+// 1.53 -> 0.25 ms.
 //
 // Data written by one CTA and read by another inside the launch (phases,
 // OTFs and seeds, fields, dL/dphi) is published by the writer's barrier,

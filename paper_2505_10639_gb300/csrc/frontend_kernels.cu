@@ -85,12 +85,12 @@ cudaError_t launch_persistent_front(Kern kern, int threads, size_t smem, long lo
 // deviations are some 10 % of it, it rounds them at its own size, and the error
 // of the other elements is 1.5e-6 to 2e-6 of their norm instead of 2e-7.
 //   HBM is the floor (frames in, spectra out); what bounds it is the latency
-// of the patch's loads and the exchanges at 16 - 18 warps per SM. With two or
-// four lanes per line, whole lines in registers and the patch staged in shared
-// memory it took, for 20 frames of two objects, 258 us at 48 px (961
-// patches), 212 us at 64 px (961, stride 29), 608 us at 96 px (441) and 250 us
-// at 128 px (225); now 131, 190, 234 and 205 us, 2.1 - 2.5 TB/s. A field too
-// small to fill the chip takes the same time either way (18.5 us, 9 patches).
+// of the patch's loads and the exchanges at 16 - 27 warps per SM. With one or
+// two lanes per line, whole lines in registers and the patch staged in shared
+// memory it took, for 12 frames of two objects, 257 us at 48 px (961
+// patches), 210 us at 64 px (961, stride 29), 604 us at 96 px (441) and 249 us
+// at 128 px (225); now 128, 188, 233 and 206 us, 2.2 - 2.5 TB/s. A field too
+// small to fill the chip takes the same time either way (17 us, 9 patches).
 template <int N>
 constexpr int kFrontMinCtas = N == 128 ? 2 : N == 96 ? 4 : N == 64 ? 6 : 9;
 

@@ -22,11 +22,13 @@ namespace {
 using namespace lanepass;
 
 // CTAs per SM that the register budget is set for: two to three times 8 warps
-// at 80-128 registers a thread. Timed with one more and one less at each size
-// (forward / adjoint / recomputing adjoint, ms): 12,800 units of 128 px 0.735 /
-// 0.842 / 1.06 with 2 (0.787 / 1.018 / 1.23 with 3); 2,904 units of 96 px 0.111
-// / 0.131 / 0.165 with 3, 4, 3 (0.117 / 0.147 / 0.170 with 4, 3, 4); 48 px 0.193
-// / 0.215 with 12 (0.196 / 0.228 with 9).
+// at 80-128 registers a thread. Timed with one more or one less at each size
+// (forward / adjoint / recomputing adjoint, ms): 12,800 units of 128 px 0.668 /
+// 0.868 / 1.002 with 2 (0.948 / 1.148 / 1.533 with 3); 2,904 units of 96 px
+// 0.107 / 0.129 / 0.161 with 3, 4, 3 (0.111 / 0.146 / 0.164 with 4, 3, 4); 6,750
+// units of 64 px 0.101 / 0.128 with 6 (0.102 / 0.132 with 5), 23,064 units 0.333
+// / 0.414 (0.326 / 0.411); 23,064 units of 48 px 0.193 / 0.214 with 12 (0.195 /
+// 0.226 with 9).
 template <int N, bool ADJ, bool RECOMPUTE>
 constexpr int kMinCtas = N == 128 ? 2 : N == 96 ? (ADJ && !RECOMPUTE ? 4 : 3) : N == 64 ? 6 : 12;
 

@@ -28,9 +28,10 @@
 // (a 128-point line is some 3,400 lane instructions and 4 KB of shared-memory
 // traffic). Measured against one or two lanes a line (64 registers of data a
 // lane, 8-12 warps an SM, stalled on instruction fetch), forward + adjoint:
-// 2,904 units of 96 px 0.404 + 0.519 -> 0.111 + 0.131 ms; 12,800 units of
-// 128 px with the field recomputed 1.95 + 2.74 -> 0.66 + 1.06 ms, kept
-// 2.68 + 2.74 -> 0.73 + 0.84 ms; 23,064 units of 64 px 0.350 + 0.458 ms.
+// 2,904 units of 96 px 0.402 + 0.508 -> 0.107 + 0.129 ms; 12,800 units of
+// 128 px with the field recomputed 1.95 + 2.74 -> 0.60 + 1.00 ms, kept
+// 2.68 + 2.64 -> 0.67 + 0.87 ms; 23,064 units of 64 px 1.35 + 1.07 -> 0.33 +
+// 0.41 ms.
 #pragma once
 
 #include <cstdint>

@@ -1,8 +1,8 @@
 // Line transforms held by one lane (N <= 64) or a lane pair (N = 96, 128), for
-// the field front end and the dictionary model: a line of N points is held by
-// S = 1 or 2 lanes, L = N / S points each; a register FFT of L points on the
-// decimated samples x[S n + s] of each lane s and, for S = 2, one radix-2 stage
-// across the lane pair by shuffles, leaving X[s L + k] in lane s.
+// the patch images of the mosaic and the aligned 64 px spectra: a line of N
+// points is held by S = 1 or 2 lanes, L = N / S points each; a register FFT of L
+// points on the decimated samples x[S n + s] of each lane s and, for S = 2, one
+// radix-2 stage across the lane pair by shuffles, leaving X[s L + k] in lane s.
 #pragma once
 
 #include <cstdint>
@@ -15,7 +15,6 @@ namespace linefft {
 
 using fftreg::cadd;
 using fftreg::cconj;
-using fftreg::cmul;
 using fftreg::cscale;
 using fftreg::csub;
 
@@ -28,13 +27,6 @@ struct Geo {
     static constexpr int THREADS = LINES * S;
 };
 
-// Barrier of the threads that work on one unit.
-struct CtaBar {
-    __device__ __forceinline__ void operator()() const { __syncthreads(); }
-};
-struct WarpBar {  // a group of one warp (32 lines per round, N <= 64)
-    __device__ __forceinline__ void operator()() const { __syncwarp(); }
-};
 __device__ __forceinline__ float2 shfl_xor2(float2 v, int m) {
     return make_float2(__shfl_xor_sync(0xffffffffu, v.x, m), __shfl_xor_sync(0xffffffffu, v.y, m));
 }

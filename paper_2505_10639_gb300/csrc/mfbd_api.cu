@@ -264,7 +264,10 @@ void release(mfbd_plan* p) {
 // boxes fit) or the caller asked for the pass machine's three kernels. The
 // other 64 px plans (more than 12 frames, boxes over 37 px) run the general
 // sizes' kernels: 6,750 units of 15 frames, forward + reduction + adjoint 0.148
-// + 0.068 + 0.133 ms on the pass machine, 0.100 + 0.075 + 0.138 on those.
+// + 0.070 + 0.133 ms on the pass machine, 0.101 + 0.073 + 0.128 on those; few
+// frames on wide boxes, evaluations of 200 patches: 40 px 6 frames 135 -> 106 us,
+// 48 px 2 frames 120 -> 89, 64 px 1 frame 146 -> 118 (900 patches 324 -> 305, the
+// least gain of 64 such plans).
 bool fused_or_split(const mfbd_plan_desc* d) {
     if (d->flags & MFBD_FLAG_SPLIT_PASSES) return true;
     int box = 1;
