@@ -104,6 +104,7 @@ __global__ void __launch_bounds__(2 * N, kFrontMinCtas<N>) spectra_kernel(const 
     float2* E = table + lane8::Twiddles<N>::kElems;
     __shared__ float win[N];
     __shared__ double red[W];
+    __shared__ float mean;  // warp 0's
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     lane8::load_twiddles<N>(table, t, 32 * W);
     window_to_smem(win, N, prm.border);
@@ -140,6 +141,7 @@ __global__ void __launch_bounds__(2 * N, kFrontMinCtas<N>) spectra_kernel(const 
         double tot = 0.0;
         for (int i = 0; i < W; ++i) tot += red[i];
         const float m = (float)(tot / (N * N));
+        if (t == 0) mean = m;
         {
             const lane8::LaneTwiddles<N> tw(table, rl.t);
 #pragma unroll
@@ -199,7 +201,7 @@ __global__ void __launch_bounds__(2 * N, kFrontMinCtas<N>) spectra_kernel(const 
                                 const float2 x = z[8 * q + c], y = E[(ky ? N - ky : 0) * S];
                                 D[ky * NH + N / 2] = make_float2(0.5f * (x.y + y.y), 0.5f * (y.x - x.x));
                                 z[8 * q + c] = make_float2(0.5f * (x.x + y.x), 0.5f * (x.y - y.y));
-                                if (ky == 0) z[8 * q + c].x += m * (float)(N * N);  // the mean's transform
+                                if (ky == 0) z[8 * q + c].x += mean * (float)(N * N);  // the mean's transform
                             }
             }
 #pragma unroll
